@@ -584,6 +584,24 @@ int rt_create(const rt_mesh_desc *m_in, const rt_params *p, void *stream, rt_sta
   CK(upload(s, &s->d_volume, vol_int));
   CK(upload(s, &s->d_dir64, dir64));
   CK(upload(s, &s->d_wt64, wt64));
+  {
+    std::vector<double> mom((size_t)(A / 2) * rt::kMomTab, 0.0);
+    for (int p = 0; p < A / 2; ++p) {
+      const double wa = m->angle_w[p], wb = m->angle_w[p + A / 2];
+      const bool sw = wb > wa;
+      const double *d = m->angle_dir + 3 * (sw ? p + A / 2 : p), w = sw ? wb : wa;
+      double *t = &mom[(size_t)p * rt::kMomTab];
+      t[0] = (sw ? wa : wb) / w;
+      t[1] = w;
+      t[11] = sw ? 1.0 : 0.0;
+      for (int k = 0; k < 3; ++k) t[2 + k] = w * d[k];
+      for (int k = 0; k < 3; ++k) t[5 + k] = w * d[k] * d[k];
+      t[8] = w * d[0] * d[1];
+      t[9] = w * d[0] * d[2];
+      t[10] = w * d[1] * d[2];
+    }
+    CK(upload(s, &s->d_mom, mom));
+  }
   CK(upload(s, &s->d_angle_of, angle_of));
   {
     std::vector<int32_t> pos_of(angle_of.size());
@@ -1369,7 +1387,7 @@ void rt_destroy(rt_state *s) {
   if (s->d_adj_stage) cudaFree(s->d_adj_stage);
   void *bufs[] = {s->d_hface, s->d_hslot, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
                   s->d_gd, s->d_kind, s->d_aux, s->d_bc_row, s->d_I0, s->d_ext, s->d_dir, s->d_wt,
-                  s->d_dir64, s->d_wt64, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
+                  s->d_dir64, s->d_wt64, s->d_mom, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
                   s->d_scratch, s->d_out16};
   for (void *b : bufs)
     if (b) cudaFree(b);

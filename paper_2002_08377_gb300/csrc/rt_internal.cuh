@@ -40,6 +40,11 @@ enum : unsigned {
   ST_CFL = 4u,  // a cell's current volume is below dt max_a sum_f max(u, 0) (gcl states)
 };
 
+// Moment coefficients of a pair from its angle with the larger weight w and
+// direction n: the other weight over w, w, w n (3), w n n (xx, yy, zz, xy, xz,
+// yz), 1 if that angle is the antipode p + A/2 (else 0).
+constexpr int kMomTab = 12;
+
 // The step kernel works on blocks of CPB consecutive (internal) cells.
 constexpr int CPB = 32;
 // Face slots of one block of CPB cells that the float QuadMap kernel stages
@@ -232,6 +237,7 @@ struct rt_state {
   void *d_wt = nullptr;        // [A/2][2] weights of the pairs (p, p + A/2)
   double *d_dir64 = nullptr;   // [A][3] double, internal angle order
   double *d_wt64 = nullptr;    // [A], internal angle order
+  double *d_mom = nullptr;     // [A/2][kMomTab] moment coefficients of the pairs (rt_moments)
   int32_t *d_angle_of = nullptr;  // internal angle position -> caller angle
   int32_t *d_pos_of = nullptr;    // caller angle -> internal angle position
   void *d_I[2] = {nullptr, nullptr};
