@@ -58,20 +58,17 @@ int cuda_fail(rt_state *s, cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail((s), e_, #call); \
   } while (0)
 
-template <typename T> cudaError_t dalloc(rt_state *s, T **p, size_t count) {
-  *p = nullptr;
-  if (count == 0) count = 1;
-  cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
-  if (e == cudaSuccess) s->device_bytes += count * sizeof(T);
-  return e;
-}
-
 cudaError_t dalloc_bytes(rt_state *s, void **p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(p, bytes);
   if (e == cudaSuccess) s->device_bytes += bytes;
   return e;
+}
+
+template <typename T> cudaError_t dalloc(rt_state *s, T **p, size_t count) {
+  if (count == 0) count = 1;
+  return dalloc_bytes(s, (void **)p, count * sizeof(T));
 }
 
 // Interleave the bits of a 21-bit integer with two zero bits.
@@ -692,6 +689,8 @@ int rt_create(const rt_mesh_desc *m_in, const rt_params *p, void *stream, rt_sta
   if (pe == cudaSuccess) pe = cudaStreamSynchronize(s->stream);
   if (s->precision == RT_FP64) cudaFree(fslot);
   CK(pe);
+  // after every other allocation: the table is left out where memory is short
+  if (s->precision == RT_FP64 && !s->moving) CK(rt::build_kout(s));
 #undef CK
   s->dt_max = kmax > 0 ? 1.0 / kmax : INFINITY;
   *out = s;
@@ -1385,7 +1384,7 @@ void rt_destroy(rt_state *s) {
     if (s->d_adj[k]) cudaFree(s->d_adj[k]);
   if (s->d_adj_ws) cudaFree(s->d_adj_ws);
   if (s->d_adj_stage) cudaFree(s->d_adj_stage);
-  void *bufs[] = {s->d_hface, s->d_hslot, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
+  void *bufs[] = {s->d_hface, s->d_hslot, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_kout, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
                   s->d_gd, s->d_kind, s->d_aux, s->d_bc_row, s->d_I0, s->d_ext, s->d_dir, s->d_wt,
                   s->d_dir64, s->d_wt64, s->d_mom, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
                   s->d_scratch, s->d_out16};

@@ -510,7 +510,7 @@ __device__ __forceinline__ void group_tile_body(const GroupArgs<R> &a, const Ste
     __syncthreads();  // the block's stage has landed
     step::face_sum<R, M, false, true, step::TRANSPORT_FORWARD>(
         reinterpret_cast<const typename SlotOf<R>::type *>(stage.slot), stage.nbr, t.wface,
-        t.uface, t.half, k0, k1, t.I_in, t.row, sub, nx, ny, nz, Ia, Ib, acca, accb, np);
+        t.uface, t.half, k0, k1, t.I_in, t.row, sub, nx, ny, nz, Ia, Ib, acca, accb, np, nullptr);
     const R dtv = t.dt_r * t.inv_vol[c];
 #pragma unroll
     for (int j = 0; j < PPT; ++j) {

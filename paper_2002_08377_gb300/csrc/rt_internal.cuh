@@ -89,6 +89,7 @@ template <typename R> struct StepArgs {
   const typename SlotOf<R>::type *slot;  // [nnz]
   const SlotF *slot_nb;     // [nnz] float static meshes: (s, neighbour index bits)
   const double *uface;      // [nnz][A/2] double states: flux coefficient of pair p through slot k
+  const double *kout;       // [N][A] double states, static meshes: sum_f max(u, 0) in row layout, or NULL
   const R *inv_vol;         // [N]
   const double *wface;      // [nnz] A_f w_f . n_f of double slots (moving meshes)
   const GasStatic *gs;      // [N]
@@ -201,6 +202,9 @@ struct rt_state {
   void *d_slot = nullptr;
   rt::SlotF *d_slot_nb = nullptr;  // float, static mesh: slot with the neighbour in w
   double *d_uface = nullptr;  // double: [nnz][A/2] flux coefficients, built once (build_uface)
+  // double, static mesh: [N][A] sum_f max(u, 0) per cell and angle (build_kout);
+  // NULL when the device had no room for it (the kernels then sum it)
+  double *d_kout = nullptr;
   // van Leer integrator: reconstruction geometry ([nnz][8] and [N][8] reals
   // of the state precision, see build_recon), stage-1 intensities [N][RS]
   // and their limited gradients [3][N][RS] (x, y, z rows in the row layout)
@@ -270,6 +274,7 @@ struct StepIO {
   bool src_only, commit;
 };
 cudaError_t launch_step_io(rt_state *s, double dt, const StepIO &io);
+cudaError_t launch_step_io64(rt_state *s, double dt, const StepIO &io);  // double states (rt_step64.cu)
 // Transport only (rt_transport.cu), rows `in` -> `out` (stride row_stride):
 // adjoint = false: I* = I - dt/V sum_f u I_up; adjoint = true: the
 // transposed operator, from rows L = dt/V lambda to M^T lambda.
@@ -283,6 +288,9 @@ cudaError_t launch_group_step(rt_state *s, double dt, const void *In, void *Out)
 cudaError_t launch_step_vl(rt_state *s, double dt);
 // Double states: fills d_uface (allocates it on first use).
 cudaError_t build_uface(rt_state *s);
+// Double states on static meshes: fills d_kout from d_uface; without room for
+// it d_kout stays NULL (no error).
+cudaError_t build_kout(rt_state *s);
 
 // A CUDA driver function by name (through the runtime's entry-point query,
 // so the library does not link the driver library itself), or NULL.

@@ -42,24 +42,27 @@ __device__ __forceinline__ double2 psub(double2 a, double2 b) {
 // Reciprocal.  Float: the PTX approximate reciprocal (one MUFU operation,
 // relative error below 2^-22, inside the float state's error budget; the
 // arguments are Gamma^k (1 + x Gamma) and 1 + dt cbar rho kappa S_G, normal
-// floats, so flushing subnormals changes nothing).  Double: that estimate
-// refined by two Newton steps r <- r (2 - x r) (about 1 ulp) where x and
-// 1/x are normal floats (|x| in [2^-125, 2^126)); any other x (physical
-// units make dt/V or cbar A far from 1) takes the IEEE double division.
+// floats, so flushing subnormals changes nothing).  Double: the PTX
+// approximate double reciprocal (no conversion to float and back) refined by
+// one third-order step r <- r (1 + e + e^2), e = 1 - x r: 3 FMAs instead of the
+// 4 of two Newton steps.  The estimate's relative error measured 9.9e-7 at
+// most over 2^28 arguments, so e^3 ~ 1e-18 stays below the final rounding
+// (0.51 ulp).  Arguments whose exponent is near the ends of the range take the
+// IEEE division.
 __device__ __forceinline__ float rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ double rcp(double x) {
-  // |x| in [2^-125, 2^126) <=> biased exponent in [898, 1149), tested on the
+  // |x| in [2^-1000, 2^1001) <=> biased exponent in [23, 2024), tested on the
   // integer pipe (the FP64 pipe is the double kernels' bottleneck)
   const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-  if (ex - 898u >= 251u) return 1.0 / x;
-  double r = (double)rcp((float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return r;
+  if (ex - 23u >= 2001u) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 template <typename R> __device__ __forceinline__ pair_t<R> prcp(pair_t<R> v) {
   return mk(rcp(v.x), rcp(v.y));
@@ -147,7 +150,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // bound g / beta.  The iteration stops when an iterate fails to decrease or
 // moves by at most `tol` of itself.  Returns 1 if it did not converge.
 __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double qdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ double qdiv(double a, double b) { return a * rcp(b); }
 
 template <typename T_>
 __device__ __forceinline__ int quartic_root(T_ alpha, T_ beta, T_ g, T_ T0, T_ tol, int max_iter,

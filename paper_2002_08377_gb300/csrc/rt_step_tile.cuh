@@ -256,11 +256,71 @@ __device__ __forceinline__ void face_sum_quads(const SlotF *__restrict__ slot,
   }
 }
 
+// face_sum of a double state on a static mesh.  u of angle p is d (tabulated)
+// and of its antipode -d, so through each face one angle of the pair enters
+// the cell and the other leaves it.  Only one of the two needs the
+// neighbour's value (MODE forward: the entering one, adjoint: the leaving
+// one); the other's terms are |d| times the cell's own value, and their sum
+// over the faces, K = sum_f max(u, 0), is static (StepArgs::kout; the same for
+// both modes).  That is one FP64 FMA per pair and face instead of two, which is
+// what bounds the double kernels (GB300 issues a warp's DFMA over 64 cycles of
+// its scheduler; the selects run on the integer pipe beside it):
+//   forward  sum u I_up           = K I - sum_in |d| I_nbr,
+//   adjoint  sum_out u (L - L_nbr) = K L - sum_out |d| L_nbr.
+// krow NULL (no memory for the table): K is summed here.
+template <typename M, int MODE>
+__device__ __forceinline__ void face_sum_static64(const int32_t *__restrict__ nbr,
+                                                  const double *__restrict__ uface, int H,
+                                                  int64_t k0, int64_t k1,
+                                                  const double *__restrict__ I_in, int RS, int sub,
+                                                  const double *__restrict__ krow,
+                                                  const double (&Ia)[M::PPT],
+                                                  const double (&Ib)[M::PPT],
+                                                  double (&acca)[M::PPT],
+                                                  double (&accb)[M::PPT], int np) {
+  constexpr int PPT = M::PPT;
+  double Ka[PPT], Kb[PPT];
+  if (!krow) {
+#pragma unroll
+    for (int j = 0; j < PPT; ++j) Ka[j] = Kb[j] = 0.0;
+    for (int64_t k = k0; k < k1; ++k)
+#pragma unroll
+      for (int j = 0; j < PPT; ++j)
+        if (M::FULL || j < np) {
+          const double d = uface[(size_t)k * H + M::pair(j, sub)];
+          Ka[j] += fmax(d, 0.0);
+          Kb[j] += fmax(-d, 0.0);
+        }
+  }
+#pragma unroll 2
+  for (int64_t k = k0; k < k1; ++k) {
+    double vx[PPT], vy[PPT];
+    M::load(I_in + (size_t)nbr[k] * RS, sub, vx, vy, np);
+#pragma unroll
+    for (int j = 0; j < PPT; ++j)
+      if (M::FULL || j < np) {
+        const double d = uface[(size_t)k * H + M::pair(j, sub)];
+        const bool b = positive(d) == (MODE == TRANSPORT_FORWARD);  // the antipode's term
+        const double ad = __hiloint2double(__double2hiint(d) & 0x7fffffff, __double2loint(d));
+        const double t = fma(-ad, b ? vy[j] : vx[j], b ? accb[j] : acca[j]);
+        acca[j] = b ? acca[j] : t;
+        accb[j] = b ? t : accb[j];
+      }
+  }
+  if (krow) M::load(krow, sub, Ka, Kb, np);
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    acca[j] = fma(Ka[j], Ia[j], acca[j]);
+    accb[j] = fma(Kb[j], Ib[j], accb[j]);
+  }
+}
+
 // sum_f u I_up over the slots [k0, k1) of one cell, neighbour rows read
 // through nbr[k] (L1/L2 serve the reuse between neighbouring cells; cells are
 // in Morton order).  slot / nbr point either to global memory or to the
 // block's copy in shared memory (K = int); PACKED: static float slots carry
-// the neighbour index in their w word and nbr is not read.
+// the neighbour index in their w word and nbr is not read.  krow: the cell's
+// row of StepArgs::kout (static double states) or NULL.
 template <typename R, typename M, bool MOVING, bool PACKED, int MODE, typename S, typename K>
 __device__ __forceinline__ void face_sum(const S *__restrict__ slot, const int32_t *__restrict__ nbr,
                                          const double *__restrict__ wface,
@@ -269,9 +329,12 @@ __device__ __forceinline__ void face_sum(const S *__restrict__ slot, const int32
                                          const R (&nx)[M::PPT], const R (&ny)[M::PPT],
                                          const R (&nz)[M::PPT], const R (&Ia)[M::PPT],
                                          const R (&Ib)[M::PPT], R (&acca)[M::PPT],
-                                         R (&accb)[M::PPT], int np) {
+                                         R (&accb)[M::PPT], int np,
+                                         const R *__restrict__ krow) {
   constexpr int PPT = M::PPT;
-  if constexpr (M::QUAD) {
+  if constexpr (sizeof(R) == 8 && !MOVING) {
+    face_sum_static64<M, MODE>(nbr, uface, H, k0, k1, I_in, RS, sub, krow, Ia, Ib, acca, accb, np);
+  } else if constexpr (M::QUAD) {
     face_sum_quads<M, MOVING, PACKED, MODE>(slot, nbr, k0, k1, I_in, RS, sub, nx, ny, nz, Ia, Ib,
                                             acca, accb);
   } else {

@@ -42,11 +42,13 @@ __device__ __forceinline__ void tile_transport(const StepArgs<R> &a, const int64
     __syncthreads();  // the block's stage has landed
     face_sum<R, M, MOVING, !MOVING, MODE>(
         reinterpret_cast<const typename SlotOf<R>::type *>(stage.slot), stage.nbr, a.wface,
-        a.uface, a.half, k0, k1, a.I_in, RS, sub, nx, ny, nz, Ia, Ib, acca, accb, np);
+        a.uface, a.half, k0, k1, a.I_in, RS, sub, nx, ny, nz, Ia, Ib, acca, accb, np, nullptr);
   } else {
     face_sum<R, M, MOVING, false, MODE>(a.slot, a.nbr, a.wface, a.uface, a.half, a.ptr[c],
                                         a.ptr[c + 1], a.I_in, RS, sub, nx, ny, nz, Ia, Ib, acca,
-                                        accb, np);
+                                        accb, np,
+                                        reinterpret_cast<const R *>(
+                                            a.kout ? a.kout + (size_t)c * RS : nullptr));
   }
   const R dtv = a.dt_r * a.inv_vol[c];
   if constexpr (MODE == TRANSPORT_FORWARD) {
@@ -99,6 +101,7 @@ cudaError_t launch_tr(rt_state *s, double dt, const void *in, void *out) {
   a.slot = reinterpret_cast<const typename SlotOf<R>::type *>(s->d_slot);
   a.slot_nb = s->d_slot_nb;
   a.uface = s->d_uface;
+  a.kout = s->d_kout;
   a.inv_vol = reinterpret_cast<const R *>(s->d_inv_vol);
   a.wface = s->d_wface;
   a.dir = reinterpret_cast<const R *>(s->d_dir);
