@@ -560,6 +560,23 @@ int rt_create(const rt_mesh_desc *m_in, const rt_params *p, void *stream, rt_sta
                  s->max_block_slots <= rt::STAGE_SLOTS)
                     ? 32 * (A / 32)
                     : 0;
+  if (s->quad_end > 0) {
+    const int Q = A / 4;
+    std::vector<float> qd(10 * (size_t)Q);
+    for (int k = 0; k < Q; ++k)
+      for (int h = 0; h < 2; ++h) {
+        const int a = 2 * k + h;  // the quad's angle, its antipode a + A/2
+        for (int d = 0; d < 2; ++d) qd[4 * k + 2 * d + h] = (float)m->angle_dir[3 * a + d];
+        qd[4 * (Q + k) + h] = (float)m->angle_dir[3 * a + 2];
+        qd[4 * (Q + k) + 2 + h] = (float)m->angle_w[a];
+        qd[8 * Q + 2 * k + h] = (float)m->angle_w[a + A / 2];
+      }
+    const cudaError_t e = upload(s, &s->d_qdir, qd);
+    if (e != cudaSuccess) return bail(cuda_fail(s, e, "direction table"));
+  }
+  s->w_uni = m->angle_w[0];
+  s->w_uniform = true;
+  for (int a = 1; a < A; ++a) s->w_uniform = s->w_uniform && m->angle_w[a] == s->w_uni;
   // dense rows (padding the quad rows to whole 128-byte lines measured no gain)
   s->row_stride = A;
   const size_t RS = (size_t)s->row_stride;
@@ -1386,7 +1403,7 @@ void rt_destroy(rt_state *s) {
   if (s->d_adj_stage) cudaFree(s->d_adj_stage);
   void *bufs[] = {s->d_hface, s->d_hslot, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_kout, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
                   s->d_gd, s->d_kind, s->d_aux, s->d_bc_row, s->d_I0, s->d_ext, s->d_dir, s->d_wt,
-                  s->d_dir64, s->d_wt64, s->d_mom, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
+                  s->d_dir64, s->d_wt64, s->d_qdir, s->d_mom, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
                   s->d_scratch, s->d_out16};
   for (void *b : bufs)
     if (b) cudaFree(b);

@@ -101,6 +101,8 @@ template <typename R> struct StepArgs {
   double *ext;              // [N][4]
   const R *dir;             // [A][4] (x, y, z, 0), caller angle order
   const R *wt2;             // [A/2][2] (w_p, w_{p+A/2})
+  int32_t w_uniform;        // 1: every angle has the weight w_uni
+  R w_uni;
   const R *I_in;            // [N][A]
   R *I_out;                 // [N][A]
   R *cellv;                 // [N][4] (v_x, v_y, v_z, e - rho v^2 / 2)
@@ -239,6 +241,9 @@ struct rt_state {
   void *d_cellv = nullptr;  // [N][4] in the state precision
   void *d_dir = nullptr;       // [A][4], caller angle order
   void *d_wt = nullptr;        // [A/2][2] weights of the pairs (p, p + A/2)
+  bool w_uniform = false;      // every angle has the weight w_uni
+  double w_uni = 0.0;
+  float *d_qdir = nullptr;     // quad rows: the direction table of step::QuadDir
   double *d_dir64 = nullptr;   // [A][3] double, internal angle order
   double *d_wt64 = nullptr;    // [A], internal angle order
   double *d_mom = nullptr;     // [A/2][kMomTab] moment coefficients of the pairs (rt_moments)

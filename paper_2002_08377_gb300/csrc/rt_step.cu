@@ -3,40 +3,39 @@
 // emitter cells (Sec. 2.5), one kernel per step.
 //
 // Layout: the intensity row of a cell stores the A/2 antipodal pairs
-// (angle p, angle p + A/2) side by side.  The flux coefficient of the
-// antipode through a face is u(p + A/2) = -(n_p . s) - w, so one dot product
-// serves both angles; on a static mesh exactly one of the two is inflow.
+// (angle p, angle p + A/2) together.  The flux coefficient of the antipode
+// through a face is u(p + A/2) = -(n_p . s) - w, so one dot product serves both
+// angles; on a static mesh exactly one of the two is inflow.
 //
-// Block = 32 cells x 8 threads.  Which pairs a thread owns is a policy:
-//   PairMap  thread `sub` owns pairs sub + 8 j (j < PPT), one 8-byte (float)
-//            or 16-byte (double) access each -- any A;
-//   QuadMap  float rows with A a multiple of 16: thread `sub` owns the pair
-//            quads sub + 8 i (one 16-byte access each, so a cell's 8 threads
-//            read 128 contiguous bytes of a neighbour row per instruction)
-//            and, when A/2 is not a multiple of 16, the pair 16 Q4 + sub.
-// The neighbour-row gathers of the face loop are bound by the L1 data pipe
-// (one wavefront per cache line an instruction touches), so wider per-thread
-// accesses cut the face loop's cost directly.  The float kernel with QuadMap
-// also copies the block's face slots and neighbour indices into shared
-// memory at its start.  Registers are capped so that 1024 threads share an
-// SM (768 for more than 5 pairs per thread).
-// Phases:
-//   A  all threads: transport over the cell's faces in slot order (no
-//      atomics, deterministic), comoving weights and the angular sums of
-//      Eq. (Jcom); each cell's 8 lanes reduce with shuffles;
-//   B  the gas temperature quartic: the float root in all 8 lanes of the
-//      cell, then, between two block barriers, one lane per cell refines it
-//      by Newton in double (with float_quartic = 1 the float root is final:
-//      no barrier);
-//   C  all threads: new intensities, store, radiation change per cell;
-//   D  after a block barrier, one lane per cell (first CPB / 32 warps): gas energy /
-//      momentum (or tally) update in double (Eqs. gas1, gas2).
-// The double-precision work is lane-per-cell because GB300's FP64 rate is a
-// small fraction of its FP32 rate.
+// quad_step_kernel (rows in the quad layout: A a multiple of 16, A >= 32) is the
+// production kernel; step_kernel (rt_step_tile.cuh's PairMap) takes every other
+// row.  Block = 32 cells x 8 threads.  Phases:
+//   transport  all threads: the cell's faces in slot order (no atomics,
+//      deterministic);
+//   A  comoving weights and the angular sums of Eq. (Jcom), reduced over the
+//      cell's 8 threads with shuffles;
+//   B  the gas temperature quartic (source_q_fast), in every lane of the cell;
+//   C  new intensities, store, radiation change per cell;
+//   D  after the block's one barrier, one lane per cell: gas energy / momentum
+//      (or tally) update in double (Eqs. gas1, gas2), on a warp that rotates
+//      with the block.
+// What bounds it: latency.  A block's time is the sum of its phases' waits (its
+// stage, the gathers of the neighbour rows from L1 / L2, the double gas update),
+// which four resident blocks overlap only in part: no unit is saturated (96^3 x
+// 64: issue 52 %, L1 data pipe 60 %, DRAM 26 %).  Hence the L2 prefetch one wave
+// ahead (11 %), one block barrier only, packed FP32 on (p, p+1) throughout,
+// registers capped at 64 so that four blocks fit, and L1 given what shared memory
+// leaves.  Per step, before (double refinement between two barriers, no
+// prefetch) and now, rows bit for bit the same: 96^3 x 80 static 558 -> 493 us,
+// 128^3 x 80 1290 -> 1131, 64^3 x 96 211 -> 168, 100^3 x 48 moving 511 -> 484.
+// Staging every row a tile reads in shared memory by bulk copies (128^3 x 64:
+// 1.18 against 0.93 ms) and 4 threads a cell (the same time) did not pay.
 #include <cuda_runtime.h>
 
 #include "rt_internal.cuh"
 #include "rt_step_args.cuh"
+#include "rt_step_quad.cuh"
+#include "rt_step_source.cuh"
 
 namespace rt {
 namespace {
@@ -46,109 +45,18 @@ using namespace step;
 struct Shared {
   float sI[CPB], sG[CPB], s1[CPB];  // the sums of Eq. (Jcom) and sum w~/(1+x), unnormalised
   float q[CPB];                     // dt cbar rho (kP B + kS J) per interior cell
-  float qa[CPB], qg[CPB], qT[CPB];  // alpha, g and the float temperature root
   float dE[CPB], dF[3][CPB];        // sum w (I* - I') and sum w n (I* - I')
   unsigned bad[CPB];
 };
 
-// The temperature equation of a float state's cell in float: the
-// coefficients of source_q from the float copies of the cell's opacities and
-// the float angular sums (alpha multiplies T^(4 + beta_P) T_ref^-beta_P),
-// with rU = 1 / D and dP, dS = dt cbar rho kappa_P, kappa_s.
-struct QuarticF {
-  float alpha, gq, rU, dP, dS;
-};
-__device__ __forceinline__ QuarticF float_coeffs(const StepArgs<float> &a, float rkP, float rkJ,
-                                                 float rkS, float eint, float SI, float SG,
-                                                 float S1) {
-  QuarticF k;
-  const float dJ = a.k_dcr_f * rkJ;
-  k.dP = a.k_dcr_f * rkP;
-  k.dS = a.k_dcr_f * rkS;
-  k.rU = rcp(fmaf(dJ, SG, S1));
-  k.alpha = a.k_alpha_f * rkP * S1 * k.rU;
-  k.gq = eint + a.k_g_f * rkJ * SI * k.rU;
-  if (a.beta_P_f != 0.0f) k.alpha *= a.tref_mbP_f;
-  return k;
-}
-// Float root of the cell's equation from the pre-step temperature (returns
-// 1 if Newton did not converge).
-__device__ __forceinline__ int float_root(const StepArgs<float> &a, const QuarticF &k, float rcv,
-                                          float eint, float *T) {
-  if (a.beta_P_f == 0.0f)
-    return quartic_root(k.alpha, rcv, k.gq, eint * rcp(rcv), 1e-7f, a.newton_max_iter, T);
-  return power_root(k.alpha, 4.0f + a.beta_P_f, rcv, k.gq, eint * rcp(rcv), 1e-7f,
-                    a.newton_max_iter, T);
-}
-// The emission term q = dt cbar rho (kP(T) B(T) + kS J~) in float.
-__device__ __forceinline__ float float_q(const StepArgs<float> &a, const QuarticF &k, float T,
-                                         float SI, float SG) {
-  float dPT = k.dP;  // dP with kappa_P at T^{n+1}
-  if (a.beta_P_f != 0.0f) dPT = k.dP * powf(T / a.T_ref_f, a.beta_P_f);
-  const float B = a.a_rad_4pi_f * (T * T) * (T * T);
-  const float J = fmaf(dPT * B, SG, SI) * k.rU;
-  return fmaf(dPT, B, k.dS * J);
-}
-
-// The same as source_q in float for float states (float_quartic = 1), from
-// the float coefficients and the internal energy e - rho v^2 / 2 that the
-// previous gas update left in cellv; coefficients or an emission term
-// outside float range fall back to the double solve.
-__device__ __forceinline__ float source_q_float(const StepArgs<float> &a, int64_t c, float rkP,
-                                                float rkJ, float rkS, float rcv, float eint,
-                                                float SI, float SG, float S1, unsigned &bad) {
-  const QuarticF k = float_coeffs(a, rkP, rkJ, rkS, eint, SI, SG, S1);
-  if (!(k.gq >= 0.0f) || !(k.alpha >= 0.0f)) {
-    bad |= ST_NONFINITE;
-    return 0.0f;
-  }
-  if (isfinite(k.alpha) && isfinite(k.gq)) {
-    float T;
-    const int nc = float_root(a, k, rcv, eint, &T);
-    const float q = float_q(a, k, T, SI, SG);
-    if (isfinite(q)) {
-      if (nc) bad |= ST_NONCONV;
-      return q;
-    }
-  }
-  return (float)source_q(a, a.gs[c], a.gd[c], (double)SI, (double)SG, (double)S1, bad);
-}
-
-// q of an interior cell of a float state (float_quartic = 0), one lane per
-// cell: the float coefficients and root as in source_q_float, the root
-// refined in double by refine_root, q in float from it; where a float value
-// is not finite or the float Newton did not converge, the double solve of
-// source_q.
-__device__ __forceinline__ float source_q_refined(const StepArgs<float> &a, const GasStatic &gr,
-                                                  const GasDyn &gd, float SI, float SG, float S1,
-                                                  float eint, unsigned &bad) {
-  const QuarticF k = float_coeffs(a, gr.frkP, gr.frkJ, gr.frkS, eint, SI, SG, S1);
-  if (!(k.gq >= 0.0f) || !(k.alpha >= 0.0f)) {
-    bad |= ST_NONFINITE;
-    return 0.0f;
-  }
-  float Tf;
-  if (isfinite(k.alpha) && isfinite(k.gq) && !float_root(a, k, gr.frcv, eint, &Tf) &&
-      isfinite(Tf)) {
-    const double T = refine_root(k.alpha, a.beta_P_f, a.beta_P, gr.rcv, k.gq, Tf);
-    const float q = float_q(a, k, (float)T, SI, SG);
-    if (isfinite(q)) return q;
-  }
-  return (float)source_q(a, gr, gd, (double)SI, (double)SG, (double)S1, bad);
-}
-
-// How float states solve the temperature equation (phase B): chosen at run
-// time from StepArgs::float_quartic, or fixed by the kernel instantiation.
-enum : int { QM_RUNTIME = 0, QM_FLOAT = 1, QM_REFINE = 2 };
-
-// One block of CPB cells: phases A-D (see the top of the file).  STAGED:
-// the caller has started the copies of the tile's slots and gas records into
-// `stage`, and the face loop waits for them; otherwise slots are read from
-// global memory and the lane-per-cell threads copy the gas records into
-// `gas` themselves.
-template <typename M, bool MOVING, bool STAGED, int QM = QM_RUNTIME>
-__device__ __forceinline__ void tile_step(const StepArgs<float> &a, const int64_t tile, Shared &sh,
-                                          SharedGas *gas, const StageView &stage) {
+// One block of CPB cells of a state whose rows are in the pair layout: the
+// phases of the quad kernel, slots read from global memory, the temperature
+// refined in double by one lane per cell between two block barriers.
+template <typename M, bool MOVING>
+__global__ void __launch_bounds__(NT, min_blocks<M::PPT>()) step_kernel(const StepArgs<float> a) {
+  __shared__ Shared sh;
+  __shared__ SharedGas gas;
+  const int64_t tile = blockIdx.x;
   using R = float;
   using V = float2;
   constexpr int PPT = M::PPT;
@@ -164,16 +72,16 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &a, const int64_
   const int lp = threadIdx.x;
   const bool lpc = lp < CPB;
   const int64_t cl = tile * CPB + lp;
-  if (!STAGED && lpc && cl < a.n_cells) {
+  if (lpc && cl < a.n_cells) {
     // prefetch of the cells' gas state for phases B and D
     const char *g = reinterpret_cast<const char *>(a.gs + cl);
     const char *d = reinterpret_cast<const char *>(a.gd + cl);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      cp_async16(reinterpret_cast<char *>(&gas->gs[lp]) + 16 * k, g + 16 * k);
+      cp_async16(reinterpret_cast<char *>(&gas.gs[lp]) + 16 * k, g + 16 * k);
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-      cp_async16(reinterpret_cast<char *>(&gas->gd[lp]) + 16 * k, d + 16 * k);
+      cp_async16(reinterpret_cast<char *>(&gas.gd[lp]) + 16 * k, d + 16 * k);
   }
 
   // ---------------- phase A: transport, I* = I - dt/V sum_f u I_up
@@ -185,21 +93,10 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &a, const int64_
     acca[j] = R(0);
     accb[j] = R(0);
   }
-  if constexpr (STAGED) {
-    const int64_t kb = a.ptr[tile * CPB];
-    const int k0 = (int)(a.ptr[c] - kb), k1 = (int)(a.ptr[c + 1] - kb);
-    cp_async_wait_all();
-    __syncthreads();  // the block's stage has landed
-    if (!a.src_only)
-      face_sum<R, M, MOVING, !MOVING, TRANSPORT_FORWARD>(stage.slot, stage.nbr, a.wface, a.uface,
-                                                         a.half, k0, k1, a.I_in, RS, sub, nx, ny,
-                                                         nz, Ia, Ib, acca, accb, np, nullptr);
-  } else {
-    if (!a.src_only)
-      face_sum<R, M, MOVING, false, TRANSPORT_FORWARD>(a.slot, a.nbr, a.wface, a.uface, a.half, a.ptr[c],
-                                    a.ptr[c + 1], a.I_in, RS, sub, nx, ny, nz, Ia, Ib, acca, accb,
-                                    np, nullptr);
-  }
+  if (!a.src_only)
+    face_sum<R, M, MOVING, false, TRANSPORT_FORWARD>(
+        reinterpret_cast<const SlotF *>(a.slot), a.nbr, a.wface, a.uface, a.half, a.ptr[c],
+        a.ptr[c + 1], a.I_in, RS, sub, nx, ny, nz, Ia, Ib, acca, accb, np, nullptr);
   {
     const R dtv = a.dt_r * a.inv_vol[c];
 #pragma unroll
@@ -270,92 +167,30 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &a, const int64_
   // ---------------- phase B: temperature quartic
   R q = 0;           // dt cbar rho (kP B + kS J~) of an interior cell
   unsigned bad = 0;  // status bits of the cell
-  const GasStatic *gs_s = STAGED ? stage.gas->gs : gas->gs;
-  const GasDyn *gd_s = STAGED ? stage.gas->gd : gas->gd;
   // float_quartic: in float, in every lane
-  const bool lane_solve = QM == QM_FLOAT || (QM == QM_RUNTIME && a.float_quartic != 0);
-  if (lane_solve) {
+  if (a.float_quartic) {
     // every lane of the cell solves the cell's quartic in float (the sums
     // are already in all 8 lanes), no block barrier
     if (kind == RT_CELL_INTERIOR)
-      q = source_q_float(a, c, fkP, fkJ, fkS, fcv, eint, sI, sG, s1, bad);
-  } else if constexpr (QM == QM_REFINE) {
-    // float states (default, staged kernels): every lane of the cell finds
-    // the float root from the float coefficients (no barrier); one lane per
-    // cell then refines it by Newton in double (the FP64 temperature solve)
-    // and forms q, or, where the float solve failed, runs the whole double
-    // solve of source_q
-    float Tf = 0.0f;
-    unsigned fst = 0;  // 0: float root, 1: solve in double, 2: non-finite coefficients
-    float qa = 0.0f, qg = 0.0f;
-    if (kind == RT_CELL_INTERIOR) {
-      const QuarticF kc = float_coeffs(a, fkP, fkJ, fkS, eint, sI, sG, s1);
-      qa = kc.alpha;
-      qg = kc.gq;
-      if (!(qg >= 0.0f) || !(qa >= 0.0f))
-        fst = 2;
-      else if (!isfinite(qa) || !isfinite(qg) || float_root(a, kc, fcv, eint, &Tf) ||
-               !isfinite(Tf))
-        fst = 1;
-    }
-    if (sub == 0) {
-      sh.sI[lc] = sI;
-      sh.sG[lc] = sG;
-      sh.s1[lc] = s1;
-      sh.qa[lc] = qa;
-      sh.qg[lc] = qg;
-      sh.qT[lc] = Tf;
-      sh.bad[lc] = fst;
-    }
-    __syncthreads();
-    // the double step: lanes 0-15 of warps 0 and 1, one cell each (measured
-    // 2 % faster per step than the 32 lanes of warp 0, 3 % faster than four
-    // lanes of each of the eight warps)
-    const int rp = (threadIdx.x >> 5) * 16 + (threadIdx.x & 31);
-    const int64_t rc = tile * CPB + rp;
-    if ((threadIdx.x & 31) < 16 && rp < CPB) {
-      float ql = 0.0f;
-      unsigned bl = 0;
-      if (rc < a.n_cells && a.kind[rc] == RT_CELL_INTERIOR) {
-        const unsigned st = sh.bad[rp];
-        const GasStatic &gr = gs_s[rp];
-        if (st == 0) {
-          const double T = refine_root(sh.qa[rp], a.beta_P_f, a.beta_P, gr.rcv, sh.qg[rp],
-                                       sh.qT[rp]);
-          const QuarticF k = float_coeffs(a, gr.frkP, gr.frkJ, gr.frkS, 0.0f, sh.sI[rp],
-                                          sh.sG[rp], sh.s1[rp]);
-          ql = float_q(a, k, (float)T, sh.sI[rp], sh.sG[rp]);
-        }
-        if (st == 2) {
-          bl = ST_NONFINITE;
-        } else if (st == 1 || !isfinite(ql)) {
-          ql = (float)source_q(a, gr, gd_s[rp], (double)sh.sI[rp], (double)sh.sG[rp],
-                               (double)sh.s1[rp], bl);
-        }
+      if (!source_q_fast<false>(a, a.gs[c], sI, sG, s1, eint, q, bad)) {
+        const float2 r = source_q_slow(a, a.gs[c], a.gd[c], sI, sG, s1, eint);
+        q = r.x;
+        bad |= __float_as_uint(r.y);
       }
-      sh.q[rp] = ql;
-      sh.bad[rp] = bl;
-    }
-    __syncthreads();
-    q = sh.q[lc];
-    bad = sh.bad[lc];
   } else {
-    // float states (default, pair-map kernels): one lane per cell finds the float root from
-    // the float coefficients, refines it by Newton in double (the FP64
-    // temperature solve) and forms q from it; where the float solve fails it
-    // runs the whole double solve of source_q
+    // one lane per cell, between two block barriers
     if (sub == 0) {
       sh.sI[lc] = sI;
       sh.sG[lc] = sG;
       sh.s1[lc] = s1;
     }
-    if (!STAGED && lpc) cp_async_wait_all();
+    if (lpc) cp_async_wait_all();
     __syncthreads();
     if (lpc) {
       float ql = 0.0f;
       unsigned bl = 0;
       if (cl < a.n_cells && a.kind[cl] == RT_CELL_INTERIOR)
-        ql = source_q_refined(a, gs_s[lp], gd_s[lp], sh.sI[lp], sh.sG[lp], sh.s1[lp],
+        ql = source_q_refined(a, gas.gs[lp], gas.gd[lp], sh.sI[lp], sh.sG[lp], sh.s1[lp],
                               a.cellv[4 * cl + 3], bl);
       sh.q[lp] = ql;
       sh.bad[lp] = bl;
@@ -451,56 +286,378 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &a, const int64_
     sh.dF[2][lc] = dfz;
     sh.bad[lc] = bad | nonfinite;
   }
-  if (!STAGED && lpc) cp_async_wait_all();
+  if (lpc) cp_async_wait_all();
   __syncthreads();
 
   // ---------------- phase D: gas exchange (Eqs. gas1, gas2), one lane per cell
   if (lpc && cl < a.n_cells)
-    gas_exchange<float, MOVING>(a, cl, gs_s[lp], gd_s[lp], sh.dE[lp], sh.dF[0][lp], sh.dF[1][lp],
+    gas_exchange<float, MOVING>(a, cl, gas.gs[lp], gas.gd[lp], sh.dE[lp], sh.dF[0][lp], sh.dF[1][lp],
                                 sh.dF[2][lp], sh.bad[lp]);
 }
 
-// Resident threads per SM the register cap aims at: kernels with up to 5
-// pairs per thread fit 1024 (64 registers), wider ones 768.
-template <int PPT> constexpr int min_blocks() { return (PPT <= 5 ? 1024 : 768) / NT; }
 
-// One block per CPB cells.
-template <typename M, bool MOVING>
-__global__ void __launch_bounds__(NT, min_blocks<M::PPT>()) step_kernel(const StepArgs<float> a) {
-  __shared__ Shared sh;
-  __shared__ SharedGas gas;
-  tile_step<M, MOVING, false>(a, blockIdx.x, sh, &gas, StageView{});
+struct QuadShared {
+  float sum[4][CPB];  // phase C: sum w dI, sum w n dI
+  float q[CPB];       // power-law opacities: the emission term
+  unsigned bad[CPB];
+};
+
+// Resident threads per SM the register cap aims at.
+template <int NQ, bool TAIL, int T> constexpr int quad_blocks() {
+  return (2 * NQ + (TAIL ? 1 : 0) <= 5 ? 1024 : 768) / (CPB * T);
 }
 
-// Float kernel with the QuadMap: the block first starts the copies of its
-// slots and gas records into shared memory, then loads its own rows and
-// directions while they land (tile_step waits before the face loop).
-template <typename M, bool MOVING, int QM>
-__global__ void __launch_bounds__(NT, min_blocks<M::PPT>())
-    step_kernel_staged(const StepArgs<float> a, int cap) {
-  __shared__ Shared sh;
+// NQ quads and, with TAIL, one pair per thread; T threads per cell.  REFINE: the
+// float temperature root is refined (float_quartic = 0).
+template <int NQ, bool TAIL, int T, bool MOVING, bool REFINE>
+__global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
+    quad_step_kernel(const __grid_constant__ StepArgs<float> a, const QuadDir qd, int cap) {
+  constexpr int CW = 32 / T;  // cells per warp
+  __shared__ QuadShared sh;
   extern __shared__ __align__(128) unsigned char dyn[];
-  const StageView v = stage_at(dyn, cap, MOVING);
-  issue_stage<MOVING>(a, blockIdx.x, v);
-  tile_step<M, MOVING, true, QM>(a, blockIdx.x, sh, nullptr, v);
+  const int64_t tile = blockIdx.x;
+  const StageView stage = stage_at(dyn, cap, MOVING);
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int lc = threadIdx.x / T, sub = threadIdx.x % T;
+  const int64_t cell = tile * CPB + lc;
+  const bool live = cell < a.n_cells;
+  const int64_t c = live ? cell : a.n_cells - 1;  // dead lanes shadow the last cell
+  const int RS = a.row;
+
+  // This kernel may start while the one before it in the stream runs its last
+  // blocks (programmatic dependent launch): what no kernel writes (slots, the
+  // connectivity, kinds, directions) is loaded first, the wait comes before
+  // anything a kernel writes.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  // stage: each warp copies the slots and gas records of its own cells
+  const int64_t kb = a.ptr[tile * CPB];
+  const int64_t kc0 = a.ptr[c], kc1 = a.ptr[c + 1];
+  {
+    const int w0 = (int)(__shfl_sync(0xffffffffu, kc0, 0) - kb);
+    const int w1 = (int)(__shfl_sync(0xffffffffu, kc1, 31) - kb);
+    if (!a.src_only) {
+      const SlotF *g = (MOVING ? reinterpret_cast<const SlotF *>(a.slot) : a.slot_nb) + kb;
+      for (int i = w0 + lane; i < w1; i += 32) {
+        cp_async16(stage.slot + i, g + i);
+        if (MOVING) cp_async4(stage.nbr + i, a.nbr + kb + i);
+      }
+    }
+  }
+  const int kind = a.kind[c];
+  float2 NX[NQ], NY[NQ], NZ[NQ];
+#pragma unroll
+  for (int i = 0; i < NQ; ++i) {
+    const float4 d = __ldg(qd.xy + sub + T * i);
+    const float2 z = __ldg(reinterpret_cast<const float2 *>(qd.zw + sub + T * i));
+    NX[i] = make_float2(d.x, d.y);
+    NY[i] = make_float2(d.z, d.w);
+    NZ[i] = z;
+  }
+  const float4 *tdir = reinterpret_cast<const float4 *>(a.dir) + 2 * T * NQ + sub;
+  float tx = 0.0f, ty = 0.0f, tz = 0.0f;
+  if (TAIL) {
+    const float4 d = __ldg(tdir);
+    tx = d.x;
+    ty = d.y;
+    tz = d.z;
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  {
+    for (int i = lane; i < 6 * CW; i += 32) {
+      const int cc = warp * CW + i / 6, k = i % 6;
+      const int64_t gc = tile * CPB + cc;
+      if (gc < a.n_cells) {
+        if (k < 4)
+          cp_async16(reinterpret_cast<char *>(&stage.gas->gs[cc]) + 16 * k,
+                     reinterpret_cast<const char *>(a.gs + gc) + 16 * k);
+        else
+          cp_async16(reinterpret_cast<char *>(&stage.gas->gd[cc]) + 16 * (k - 4),
+                     reinterpret_cast<const char *>(a.gd + gc) + 16 * (k - 4));
+      }
+    }
+  }
+  // one warp prefetches the tile one wave of blocks ahead into L2, so that its
+  // gathers and its own stage find the rows there instead of waiting on HBM
+  const int64_t pc0 = (tile + kAhead) * CPB;
+  const bool ahead = warp == 1 && pc0 < a.n_cells && !a.src_only;
+  const int64_t pc1 = pc0 + CPB < a.n_cells ? pc0 + CPB : a.n_cells;
+  int64_t pk0 = 0, pk1 = 0;
+  if (ahead && lane == 0) {
+    const unsigned n = (unsigned)(pc1 - pc0);
+    pk0 = a.ptr[pc0];
+    pk1 = a.ptr[pc1];
+    l2_prefetch(a.I_in + (size_t)pc0 * RS, n * RS * (unsigned)sizeof(float));
+    l2_prefetch(a.gs + pc0, n * (unsigned)sizeof(GasStatic));
+    l2_prefetch(a.gd + pc0, n * (unsigned)sizeof(GasDyn));
+    l2_prefetch(a.cellv + 4 * pc0, n * 16);
+  }
+  const float dtv = a.dt_r * a.inv_vol[c];
+  const float4 cv = *reinterpret_cast<const float4 *>(a.cellv + 4 * c);
+  cp_async_wait_all();
+  __syncwarp();  // the warp's stage has landed
+  if (ahead && lane == 0 && pk1 > pk0)
+    l2_prefetch((MOVING ? reinterpret_cast<const SlotF *>(a.slot) : a.slot_nb) + pk0,
+                (unsigned)(pk1 - pk0) * (unsigned)sizeof(SlotF));
+
+  // ---------------- transport, I* = I - dt/V sum_f u I_up
+  float2 IA[NQ], IB[NQ], IT = bcast(0.0f);
+  {
+    const float *o = a.I_in + (size_t)c * RS;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const float4 t = reinterpret_cast<const float4 *>(o)[sub + T * i];
+      IA[i] = make_float2(t.x, t.y);
+      IB[i] = make_float2(t.z, t.w);
+    }
+    if (TAIL) IT = reinterpret_cast<const float2 *>(o)[2 * T * NQ + sub];
+  }
+  if (!a.src_only) {
+    QuadSums<NQ> u;
+    quad_faces<NQ, TAIL, T, MOVING>(stage.slot, stage.nbr, (int)(kc0 - kb), (int)(kc1 - kb),
+                                    a.I_in, RS, sub, NX, NY, NZ, tx, ty, tz, IA, IB, IT, u);
+    const float2 mdt = bcast(-dtv), pdt = bcast(dtv);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      IA[i] = pfma(mdt, u.CA[i], IA[i]);
+      IB[i] = pfma(pdt, u.CB[i], IB[i]);
+    }
+    IT = pfma(mdt, u.CT, IT);
+    if constexpr (MOVING) {
+      if (a.gcl_rate) {
+        // geometric conservation law: times V^n / V^{n+1} (see rt_step64.cu)
+        const float2 ratio = bcast(rcp(fmaf(dtv, (float)a.gcl_rate[c], 1.0f)));
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+          IA[i] = pmul(IA[i], ratio);
+          IB[i] = pmul(IB[i], ratio);
+        }
+        IT = pmul(IT, ratio);
+      }
+    }
+  }
+
+  // ---------------- phase A: Gamma = 1 -+ v.n / c (first order in v/c), w~ =
+  // w / Gamma^2 (normalised by their sum), S_I = sum w~ Gamma^4 I* / (1 + x Gamma), S_G
+  // = sum w~ Gamma / (1 + x Gamma), S_1 = sum w~ / (1 + x Gamma).  To all orders Gamma
+  // = gamma G: the weights' normalisation cancels gamma^2, so gamma enters only per
+  // cell (x -> gamma x, S_I -> gamma^4 S_I, S_G -> gamma S_G and, in phase C, q ->
+  // q / gamma^3; emitters: rate gamma, source / gamma^4).  A uniform weight cancels too.
+  const float icr = a.inv_c_r;
+  const float vx = cv.x * icr, vy = cv.y * icr, vz = cv.z * icr, eint = cv.w;
+  const int li = (int)(c - tile * CPB);
+  const GasStatic &gs = stage.gas->gs[li];
+  float xs = a.dt_cbar_r * (gs.frkJ + gs.frkS);
+  double2 ax = make_double2(0.0, 0.0);
+  if (kind != RT_CELL_INTERIOR) ax = a.aux[c];
+  if (kind == RT_CELL_EMITTER) xs = (float)(a.dt * a.cbar * ax.x);
+  const float gam = frame_gamma(a.boost, vx, vy, vz);
+  if (a.boost) xs *= gam;
+  const bool uw = a.w_uniform;
+  const float2 *W2 = reinterpret_cast<const float2 *>(a.wt2) + 2 * T * NQ + sub;  // the tail pair's
+  // the sums over a thread's angles run over its pairs in order, the first
+  // angles' (x) and the antipodes' (y) apart
+  float2 sIv = bcast(0.0f), sGv = sIv, s1v = sIv;
+  {
+    const float2 XS = bcast(xs), one = bcast(1.0f), m1 = bcast(-1.0f);
+    const float2 VX = bcast(vx), VY = bcast(vy), VZ = bcast(vz);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const float2 BN = pfma(VX, NX[i], pfma(VY, NY[i], pmul(VZ, NZ[i])));
+      const float2 GA = pfma(BN, m1, one), GB = padd(BN, one);
+      const float2 GA2 = pmul(GA, GA), GB2 = pmul(GB, GB);
+      // t = w / (Gamma^2 (1 + x Gamma)): one reciprocal per angle
+      float2 ta = prcpf(pmul(GA2, pfma(XS, GA, one))), tb = prcpf(pmul(GB2, pfma(XS, GB, one)));
+      float2 wa = bcast(a.w_uni), wb = wa;
+      if (!uw) {
+        const float4 d = __ldg(qd.zw + sub + T * i);
+        wa = make_float2(d.z, d.w);
+        wb = __ldg(qd.wb + sub + T * i);
+      }
+      ta = pmul(wa, ta);
+      tb = pmul(wb, tb);
+      const float2 ua = pmul(ta, pmul(GA2, GA2)), ub = pmul(tb, pmul(GB2, GB2));
+      s1v.x = (s1v.x + ta.x) + ta.y;
+      s1v.y = (s1v.y + tb.x) + tb.y;
+      sIv.x = fmaf(ua.y, IA[i].y, fmaf(ua.x, IA[i].x, sIv.x));
+      sIv.y = fmaf(ub.y, IB[i].y, fmaf(ub.x, IB[i].x, sIv.y));
+      sGv.x = fmaf(ta.y, GA.y, fmaf(ta.x, GA.x, sGv.x));
+      sGv.y = fmaf(tb.y, GB.y, fmaf(tb.x, GB.x, sGv.y));
+    }
+    if (TAIL) {
+      const float bn = fmaf(vx, tx, fmaf(vy, ty, vz * tz));
+      const float2 G = make_float2(1.0f - bn, 1.0f + bn), G2 = pmul(G, G);
+      const float2 w = uw ? bcast(a.w_uni) : __ldg(W2);
+      const float2 t = pmul(w, prcpf(pmul(G2, pfma(XS, G, one))));
+      s1v = padd(s1v, t);
+      sIv = pfma(pmul(t, pmul(G2, G2)), IT, sIv);
+      sGv = pfma(t, G, sGv);
+    }
+  }
+  float sI = team_sum<T>(sIv.x + sIv.y), sG = team_sum<T>(sGv.x + sGv.y),
+        s1 = team_sum<T>(s1v.x + s1v.y);
+  if (a.boost) {
+    const float g2 = gam * gam;
+    sI *= g2 * g2;
+    sG *= gam;
+  }
+
+  // ---------------- phase B: the temperature equation, in every lane of the cell
+  float q = 0.0f;  // dt cbar rho (kP B + kS J~)
+  unsigned bad = 0;
+  if (REFINE && a.beta_P_f != 0.0f) {
+    // power-law opacities: the double Newton step takes a double power, so one
+    // lane per cell runs it, between two block barriers
+    if (sub == 0) {
+      sh.sum[0][lc] = sI;
+      sh.sum[1][lc] = sG;
+      sh.sum[2][lc] = s1;
+      sh.sum[3][lc] = eint;
+    }
+    __syncthreads();
+    const int64_t cl = tile * CPB + lane;
+    if (warp == (int)(tile % T) && cl < a.n_cells) {
+      float2 r = bcast(0.0f);
+      if (a.kind[cl] == RT_CELL_INTERIOR) {
+        float ql = 0.0f;
+        unsigned bl = 0;
+        // its coefficient check; the root itself is source_q_slow's
+        if (!source_q_fast<REFINE>(a, stage.gas->gs[lane], sh.sum[0][lane], sh.sum[1][lane],
+                                   sh.sum[2][lane], sh.sum[3][lane], ql, bl))
+          r = source_q_slow(a, stage.gas->gs[lane], stage.gas->gd[lane], sh.sum[0][lane],
+                            sh.sum[1][lane], sh.sum[2][lane], sh.sum[3][lane]);
+        else
+          r = make_float2(ql, __uint_as_float(bl));
+      }
+      sh.q[lane] = r.x;
+      sh.bad[lane] = __float_as_uint(r.y);
+    }
+    __syncthreads();
+    q = sh.q[lc];
+    bad = sh.bad[lc];
+    __syncthreads();  // before sh.sum and sh.bad are written again
+  } else if (kind == RT_CELL_INTERIOR) {
+    if (!source_q_fast<REFINE>(a, gs, sI, sG, s1, eint, q, bad)) {
+      const float2 r = source_q_slow(a, gs, stage.gas->gd[li], sI, sG, s1, eint);
+      q = r.x;
+      bad |= __float_as_uint(r.y);
+    }
+  }
+
+  // ---------------- phase C: interior I' = (I* Gamma^3 + q) / (Gamma^3 (1 + x Gamma));
+  // emitter the same with x -> dt cbar (rho kappa)_src and q -> that rate times
+  // I_src (Sec. 2.5); boundary I' = I* - f (I* - I0).  The gas receives the
+  // difference of the stored intensities: the energy bookkeeping is then exact
+  // in float.
+  float dea = 0.0f, deb = 0.0f, dfx = 0.0f, dfy = 0.0f, dfz = 0.0f;
+  {
+    const bool bnd = kind == RT_CELL_BOUNDARY;
+    float2 mf = bcast(0.0f);
+    const float *I0 = a.I0;
+    if (bnd) {
+      mf = bcast(-(float)((ax.x <= a.dt) ? 1.0 : a.dt / ax.x));
+      I0 = a.I0 + (size_t)a.bc_row[c] * RS;
+    } else {
+      if (kind == RT_CELL_EMITTER) q = xs * (float)ax.y;
+      if (a.boost) q /= kind == RT_CELL_EMITTER ? (gam * gam) * (gam * gam) : gam * gam * gam;
+    }
+    const float2 QQ = bcast(q), XS = bcast(xs), one = bcast(1.0f), m1 = bcast(-1.0f);
+    float *out = a.I_out + (size_t)c * RS;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const float4 xy = load_again(qd.xy + sub + T * i), zw = load_again(qd.zw + sub + T * i);
+      float2 na, nb;
+      if (bnd) {
+        const float4 t = reinterpret_cast<const float4 *>(I0)[sub + T * i];
+        na = pfma(mf, psub(IA[i], make_float2(t.x, t.y)), IA[i]);
+        nb = pfma(mf, psub(IB[i], make_float2(t.z, t.w)), IB[i]);
+      } else {
+        const float2 BN = pfma(bcast(vx), make_float2(xy.x, xy.y),
+                               pfma(bcast(vy), make_float2(xy.z, xy.w),
+                                    pmul(bcast(vz), make_float2(zw.x, zw.y))));
+        const float2 GA = pfma(BN, m1, one), GB = padd(BN, one);
+        const float2 GA3 = pmul(pmul(GA, GA), GA), GB3 = pmul(pmul(GB, GB), GB);
+        na = pmul(pfma(IA[i], GA3, QQ), prcpf(pmul(GA3, pfma(XS, GA, one))));
+        nb = pmul(pfma(IB[i], GB3, QQ), prcpf(pmul(GB3, pfma(XS, GB, one))));
+      }
+      if (live)
+        reinterpret_cast<float4 *>(out)[sub + T * i] = make_float4(na.x, na.y, nb.x, nb.y);
+      float2 wa = bcast(a.w_uni), wb = wa;
+      if (!uw) {
+        wa = make_float2(zw.z, zw.w);
+        wb = __ldg(qd.wb + sub + T * i);
+      }
+      const float2 da = pmul(wa, psub(IA[i], na)), db = pmul(wb, psub(IB[i], nb));
+      dea = (dea + da.x) + da.y;
+      deb = (deb + db.x) + db.y;
+      const float2 df = psub(da, db);  // the antipode has direction -n
+      dfx = fmaf(xy.y, df.y, fmaf(xy.x, df.x, dfx));
+      dfy = fmaf(xy.w, df.y, fmaf(xy.z, df.x, dfy));
+      dfz = fmaf(zw.y, df.y, fmaf(zw.x, df.x, dfz));
+    }
+    if (TAIL) {
+      const float4 n = load_again(tdir);
+      float2 nt;
+      if (bnd) {
+        nt = pfma(mf, psub(IT, reinterpret_cast<const float2 *>(I0)[2 * T * NQ + sub]), IT);
+      } else {
+        const float bn = fmaf(vx, n.x, fmaf(vy, n.y, vz * n.z));
+        const float2 G = make_float2(1.0f - bn, 1.0f + bn);
+        const float2 G3 = pmul(pmul(G, G), G);
+        nt = pmul(pfma(IT, G3, QQ), prcpf(pmul(G3, pfma(XS, G, one))));
+      }
+      if (live) reinterpret_cast<float2 *>(out)[2 * T * NQ + sub] = nt;
+      const float2 w = uw ? bcast(a.w_uni) : __ldg(W2);
+      const float2 d = pmul(w, psub(IT, nt));
+      dea += d.x;
+      deb += d.y;
+      const float df = d.x - d.y;
+      dfx = fmaf(n.x, df, dfx);
+      dfy = fmaf(n.y, df, dfy);
+      dfz = fmaf(n.z, df, dfz);
+    }
+  }
+  {
+    const float v[4] = {dea + deb, dfx, dfy, dfz};
+    team_store4<T>(v, sub, lc, sh.sum);
+    if (sub == 0) sh.bad[lc] = bad;
+  }
+  __syncthreads();
+
+  // ---------------- phase D: gas exchange, one lane per cell
+  const int64_t cl = tile * CPB + lane;
+  if (warp == (int)(tile % T) && cl < a.n_cells) {
+    unsigned b = sh.bad[lane];
+    if (!isfinite(sh.sum[0][lane])) b |= ST_NONFINITE;
+    gas_exchange<float, MOVING>(a, cl, stage.gas->gs[lane], stage.gas->gd[lane], sh.sum[0][lane],
+                                sh.sum[1][lane], sh.sum[2][lane], sh.sum[3][lane], b);
+  }
 }
 
-// Launches one step with pair map M.
-template <typename M, bool MOVING, bool STAGED>
-cudaError_t launch_t(rt_state *s, double dt, const StepIO &io) {
+template <int NQ, bool TAIL, int T, bool MOVING>
+cudaError_t launch_quad(rt_state *s, double dt, const StepIO &io) {
   const StepArgs<float> a = step_args<float>(s, dt, io);
   const unsigned blocks = (unsigned)((s->n_cells + CPB - 1) / CPB);
-  if constexpr (STAGED) {
-    const int cap = stage_cap(s->max_block_slots);
-    if (a.float_quartic)
-      step_kernel_staged<M, MOVING, QM_FLOAT>
-          <<<blocks, NT, stage_bytes(cap, MOVING), s->stream>>>(a, cap);
-    else
-      step_kernel_staged<M, MOVING, QM_REFINE>
-          <<<blocks, NT, stage_bytes(cap, MOVING), s->stream>>>(a, cap);
-  } else {
-    step_kernel<M, MOVING><<<blocks, NT, 0, s->stream>>>(a);
-  }
+  const int cap = stage_cap(s->max_block_slots);
+  const float4 *xy = reinterpret_cast<const float4 *>(s->d_qdir);
+  const int Q = s->n_angles / 4;
+  const QuadDir qd{xy, xy + Q, reinterpret_cast<const float2 *>(xy + 2 * Q)};
+  const size_t sm = stage_bytes(cap, MOVING);
+  auto *k = a.float_quartic ? quad_step_kernel<NQ, TAIL, T, MOVING, false>
+                            : quad_step_kernel<NQ, TAIL, T, MOVING, true>;
+  const cudaError_t e =
+      launch_carved(k, blocks, CPB * T, sm, quad_blocks<NQ, TAIL, T>(), sizeof(QuadShared), true,
+                    s->stream, a, qd, cap);
+  if (e != cudaSuccess) return e;
+  s->launches++;
+  return cudaGetLastError();
+}
+
+template <typename M, bool MOVING>
+cudaError_t launch_pairs(rt_state *s, double dt, const StepIO &io) {
+  const StepArgs<float> a = step_args<float>(s, dt, io);
+  step_kernel<M, MOVING>
+      <<<(unsigned)((s->n_cells + CPB - 1) / CPB), NT, 0, s->stream>>>(a);
   s->launches++;
   return cudaGetLastError();
 }
@@ -509,29 +666,29 @@ template <bool MOVING, bool FULL>
 cudaError_t dispatch_pairs(rt_state *s, double dt, const StepIO &io) {
   const int ppt = (s->n_angles / 2 + KT - 1) / KT;
   switch (ppt) {
-    case 1: return launch_t<PairMap<float, 1, FULL>, MOVING, false>(s, dt, io);
-    case 2: return launch_t<PairMap<float, 2, FULL>, MOVING, false>(s, dt, io);
-    case 3: return launch_t<PairMap<float, 3, FULL>, MOVING, false>(s, dt, io);
-    case 4: return launch_t<PairMap<float, 4, FULL>, MOVING, false>(s, dt, io);
-    case 5: return launch_t<PairMap<float, 5, FULL>, MOVING, false>(s, dt, io);
-    case 6: return launch_t<PairMap<float, 6, FULL>, MOVING, false>(s, dt, io);
-    case 7: return launch_t<PairMap<float, 7, FULL>, MOVING, false>(s, dt, io);
-    case 8: return launch_t<PairMap<float, 8, FULL>, MOVING, false>(s, dt, io);
+    case 1: return launch_pairs<PairMap<float, 1, FULL>, MOVING>(s, dt, io);
+    case 2: return launch_pairs<PairMap<float, 2, FULL>, MOVING>(s, dt, io);
+    case 3: return launch_pairs<PairMap<float, 3, FULL>, MOVING>(s, dt, io);
+    case 4: return launch_pairs<PairMap<float, 4, FULL>, MOVING>(s, dt, io);
+    case 5: return launch_pairs<PairMap<float, 5, FULL>, MOVING>(s, dt, io);
+    case 6: return launch_pairs<PairMap<float, 6, FULL>, MOVING>(s, dt, io);
+    case 7: return launch_pairs<PairMap<float, 7, FULL>, MOVING>(s, dt, io);
+    case 8: return launch_pairs<PairMap<float, 8, FULL>, MOVING>(s, dt, io);
     default: return cudaErrorInvalidValue;
   }
 }
 
-// Float rows with A = 16 m (32 <= A <= 128) whose blocks' slots fit the
-// shared-memory stage: QuadMap<A / 32, A % 32 != 0>.
+// Rows in the quad layout: A = 16 m (32 <= A <= 128), m / 2 quads per thread and a
+// tail pair when m is odd.
 template <bool MOVING> cudaError_t dispatch_quads(rt_state *s, double dt, const StepIO &io) {
   switch (s->n_angles / 16) {
-    case 2: return launch_t<QuadMap<1, false>, MOVING, true>(s, dt, io);
-    case 3: return launch_t<QuadMap<1, true>, MOVING, true>(s, dt, io);
-    case 4: return launch_t<QuadMap<2, false>, MOVING, true>(s, dt, io);
-    case 5: return launch_t<QuadMap<2, true>, MOVING, true>(s, dt, io);
-    case 6: return launch_t<QuadMap<3, false>, MOVING, true>(s, dt, io);
-    case 7: return launch_t<QuadMap<3, true>, MOVING, true>(s, dt, io);
-    case 8: return launch_t<QuadMap<4, false>, MOVING, true>(s, dt, io);
+    case 2: return launch_quad<1, false, 8, MOVING>(s, dt, io);
+    case 3: return launch_quad<1, true, 8, MOVING>(s, dt, io);
+    case 4: return launch_quad<2, false, 8, MOVING>(s, dt, io);
+    case 5: return launch_quad<2, true, 8, MOVING>(s, dt, io);
+    case 6: return launch_quad<3, false, 8, MOVING>(s, dt, io);
+    case 7: return launch_quad<3, true, 8, MOVING>(s, dt, io);
+    case 8: return launch_quad<4, false, 8, MOVING>(s, dt, io);
     default: return cudaErrorInvalidValue;
   }
 }

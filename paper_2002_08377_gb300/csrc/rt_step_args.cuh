@@ -175,6 +175,8 @@ template <typename R> StepArgs<R> step_args(rt_state *s, double dt, const StepIO
   a.status = s->d_status;
   a.bad_cell = s->d_bad;
   a.kout = s->d_kout;
+  a.w_uniform = s->w_uniform;
+  a.w_uni = R(s->w_uni);
   return a;
 }
 

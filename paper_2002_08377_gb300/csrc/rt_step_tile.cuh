@@ -72,7 +72,7 @@ __device__ __forceinline__ StageView stage_at(unsigned char *base, int cap, bool
 
 // All threads: asynchronous copies of tile `tile`'s slots, neighbour indices
 // and (GAS) gas records into v (one contiguous range of each array).
-template <bool MOVING, bool GAS = true>
+template <bool MOVING, bool GAS = true, int NTH = NT>
 __device__ __forceinline__ void issue_stage(const StepArgs<float> &a, int64_t tile,
                                             const StageView &v) {
   const int64_t c0 = tile * CPB;
@@ -81,17 +81,17 @@ __device__ __forceinline__ void issue_stage(const StepArgs<float> &a, int64_t ti
   const int cnt = (int)(a.ptr[c1] - kb);
   if (MOVING) {
     const SlotF *gsl = reinterpret_cast<const SlotF *>(a.slot) + kb;
-    for (int i = threadIdx.x; i < cnt; i += NT) {
+    for (int i = threadIdx.x; i < cnt; i += NTH) {
       cp_async16(v.slot + i, gsl + i);
       cp_async4(v.nbr + i, a.nbr + kb + i);
     }
   } else {
-    for (int i = threadIdx.x; i < cnt; i += NT) cp_async16(v.slot + i, a.slot_nb + kb + i);
+    for (int i = threadIdx.x; i < cnt; i += NTH) cp_async16(v.slot + i, a.slot_nb + kb + i);
   }
   if (!GAS) return;
   // 6 x 16 bytes per cell: GasStatic (64) then GasDyn (32)
   const int nc = (int)(c1 - c0);
-  for (int i = threadIdx.x; i < 6 * nc; i += NT) {
+  for (int i = threadIdx.x; i < 6 * nc; i += NTH) {
     const int cc = i / 6, k = i % 6;
     if (k < 4)
       cp_async16(reinterpret_cast<char *>(&v.gas->gs[cc]) + 16 * k,
@@ -100,6 +100,37 @@ __device__ __forceinline__ void issue_stage(const StepArgs<float> &a, int64_t ti
       cp_async16(reinterpret_cast<char *>(&v.gas->gd[cc]) + 16 * (k - 4),
                  reinterpret_cast<const char *>(a.gd + c0 + cc) + 16 * (k - 4));
   }
+}
+
+// L2 prefetch of `bytes` (a multiple of 16) at p (16-byte aligned).
+__device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+}
+// Tiles between a block's tile and the one it prefetches: a wave of four blocks
+// on each of 152 SMs.
+constexpr int kAhead = 608;
+// Launches k with shared memory for `resident` blocks an SM (dynamic `sm` bytes
+// and `fixed` static ones each) and no more: the rest of the SM's 256 KB is L1
+// for the row gathers (the driver's split left them 121 KB: 2 % slower steps).
+// pdl: the kernel calls griddepcontrol.wait before it reads what a kernel before
+// it writes, and may start while that one ends.
+template <typename... P, typename... A>
+cudaError_t launch_carved(void (*k)(P...), unsigned blocks, int threads, size_t sm, int resident,
+                          size_t fixed, bool pdl, cudaStream_t stream, A &&...args) {
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  const size_t need = resident * (sm + fixed + 1024), all = 228 * 1024;
+  at[0].val.sharedMemCarveout = (unsigned)(need < all ? (need * 100 + all - 1) / all : 100);
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
 // ------------------------------------------------------------ pair maps
