@@ -64,8 +64,8 @@ struct alignas(32) GasDyn {
   double e, mx, my, mz;
 };
 
-// Gas dynamics (rt_hydro.cu): one record per face (caller face order) and
-// one per directed slot (internal slot order).
+// Gas dynamics (rt_hydro.cu): one record per face (numbered in the order the
+// internal cells list them first) and one per directed slot (internal slot order).
 struct HydroFace {
   int32_t i, j;        // internal cells: first (left) and second (right)
   double area;
@@ -75,8 +75,6 @@ struct HydroFace {
 struct HydroSlot {
   double own[3], nbr[3];  // face centroid minus the cell's / the neighbour image's centroid
   double area;
-  double sign;            // +1: the cell is the face's first cell, -1: its second
-  int64_t face;           // caller face index (into the face fluxes)
   double wr[3];           // least-squares weight A_f / |r|^2 times r = own - nbr (set on the device)
 };
 
@@ -259,6 +257,7 @@ struct rt_state {
   // gas dynamics (params.hydro): face and slot records, work area
   rt::HydroFace *d_hface = nullptr;
   rt::HydroSlot *d_hslot = nullptr;
+  int32_t *d_hface_id = nullptr;  // [nnz] face of the slot; ~face where the cell is its second cell
   double *d_hlsq = nullptr;  // [N][10] cofactors and determinant of each cell's normal matrix
   double *d_hwork = nullptr;
   double *d_scratch = nullptr;  // reduction partials

@@ -68,6 +68,16 @@ template <typename R> __device__ __forceinline__ pair_t<R> prcp(pair_t<R> v) {
   return mk(rcp(v.x), rcp(v.y));
 }
 
+// A double as an integer that orders like it (-0 below +0), and back: ranges
+// kept as these are compared on the integer pipe.
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double key_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+
 // Four consecutive reals (16-byte aligned for float, 32 for double).
 __device__ __forceinline__ void store4(float *p, float x, float y, float z, float w) {
   *reinterpret_cast<float4 *>(p) = make_float4(x, y, z, w);
