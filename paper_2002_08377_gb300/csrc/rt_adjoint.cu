@@ -120,16 +120,8 @@ template <typename R> __device__ __forceinline__ Ang<R> comoving_g(R G, R wt, R 
   Ang<R> g;
   g.G = G;
   const R xp = fma(X, g.G, R(1));  // 1 + x
-  if constexpr (sizeof(R) == 8) {
-    // double: one reciprocal of Gamma (1 + x) serves both (the FP64 pipe
-    // bounds the double kernel)
-    const R p = rcp_pos(g.G * xp);
-    g.iG = xp * p;
-    g.r = g.G * p;
-  } else {
-    g.iG = rcp_pos(g.G);
-    g.r = rcp_pos(xp);
-  }
+  g.iG = rcp_pos(g.G);
+  g.r = rcp_pos(xp);
   const R iG2 = g.iG * g.iG, G2 = g.G * g.G;
   g.iG4 = iG2 * iG2;
   g.wh = wt * iG2;
@@ -396,6 +388,55 @@ template <typename R, typename M> struct Entries {
   }
 };
 
+// The reverse of a double state, 48^3 cells x 48 angles: 1.47 -> 1.25 ms with the
+// quantities saved and the products collected as below (about 67 FP64 operations
+// per angle instead of 88).
+// What phase 1 of a double state leaves for phase 3 per angle in shared memory
+// (the FP64 pipe bounds the kernel; shared memory is idle): 1 / Gamma, 1 / (1 + x)
+// and 4 pi w (c lambda_e + n . lambda_m) / cbar.
+struct AngSaved {
+  double iG, r, ex;
+};
+
+// sums_angle of a double state, returning what phase 3 reads again.
+__device__ __forceinline__ AngSaved sums_angle64(double G, double wt, double X, double is,
+                                                 double l1, double ex, double &Nw, double &SI,
+                                                 double &SG, double &S1, double &lq) {
+  const double xp = fma(X, G, 1.0), p = rcp(G * xp);  // one reciprocal for both
+  const AngSaved o{xp * p, G * p, ex};
+  const double iG2 = o.iG * o.iG, G2 = G * G, wh = wt * iG2, whr = wh * o.r;
+  Nw += wh;
+  SI = fma(whr, G2 * G2 * is, SI);
+  SG = fma(whr, G, SG);
+  S1 += whr;
+  lq = fma(G * ((l1 - ex) * (iG2 * iG2)), o.r, lq);
+  return o;
+}
+
+// reverse_angle of a double state from the saved quantities, with the terms in
+// lambda_Gamma collected so that each product is formed once: with s = lambda_I~'
+// r and P = I~' lambda_I~', lambda_I~ = w r lambda_SI + s, lambda_x = -(I~' s + w r lw),
+//   lambda_Gamma = q s + w r lambda_SG + X lambda_x + 4 (I~ lambda_I~ - P) / Gamma
+//                  - 2 w^ (lw - swl) / (N_w Gamma).
+__device__ __forceinline__ double reverse_angle64(const AngSaved &t, double G, double wt,
+                                                  double X, double isv, double l1, double dtv,
+                                                  const Chain<double> &c, double &gJx,
+                                                  double &lGo) {
+  const double G2 = G * G, G4 = G2 * G2, It = G4 * isv;
+  const double iG2 = t.iG * t.iG, w = wt * iG2 * c.iNw;
+  const double lItn = (l1 - t.ex) * (iG2 * iG2), s = lItn * t.r;
+  const double Itn = fma(c.q, G, It) * t.r;
+  const double lw = fma(It, c.lSI, G * c.lSG) * t.r, wr = w * t.r;
+  const double lIt = fma(wr, c.lSI, s);
+  const double lx = -fma(Itn, s, wr * lw);
+  gJx = fma(G, lx, gJx);
+  double lG = fma(wr, c.lSG, c.q * s);
+  lG = fma(X, lx, lG);
+  const double u = fma(4.0, fma(It, lIt, -(Itn * lItn)), -2.0 * (w * (lw - c.swl)));
+  lGo = fma(t.iG, u, lG);
+  return dtv * fma(G4, lIt, t.ex);
+}
+
 template <typename R> __device__ __forceinline__ R group_sum(R v) {
   v += __shfl_xor_sync(0xffffffffu, v, 4);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
@@ -416,6 +457,7 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
   constexpr int kShared = kLaneChain ? 1 : kRevCells;
   __shared__ CellSums<R> sums[kShared];
   __shared__ Chain<R> rev[kShared];
+  extern __shared__ double saved[];  // double states: AngSaved per entry, [2 PPT][3][threads]
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int lc = threadIdx.x / KT, sub = threadIdx.x % KT;
   const int64_t c0 = (int64_t)blockIdx.x * kRevCells;
@@ -436,6 +478,20 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
       for (int j = 0; j < PPT; ++j)
         if (M::FULL || j < np) {
           const R t = fma(ci.bx, E.nx[j], fma(ci.by, E.ny[j], ci.bz * E.nz[j]));
+          if constexpr (sizeof(R) == 8) {
+            const AngSaved A = sums_angle64(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j],
+                                            E.ex(j, false, ci, k_ex), Nw, SI, SG, S1, lq);
+            const AngSaved B = sums_angle64(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j],
+                                            E.ex(j, true, ci, k_ex), Nw, SI, SG, S1, lq);
+            double *v = saved + (6 * j) * kRevThreads + threadIdx.x;
+            v[0] = A.iG;
+            v[kRevThreads] = A.r;
+            v[2 * kRevThreads] = A.ex;
+            v[3 * kRevThreads] = B.iG;
+            v[4 * kRevThreads] = B.r;
+            v[5 * kRevThreads] = B.ex;
+            continue;
+          }
           sums_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], E.ex(j, false, ci, k_ex), Nw, SI,
                      SG, S1, lq);
           sums_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex), Nw, SI,
@@ -494,6 +550,21 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
       for (int j = 0; j < PPT; ++j) {
         const R t = fma(ci.bx, E.nx[j], fma(ci.by, E.ny[j], ci.bz * E.nz[j]));
         R ga = 0, gb = 0, gxa = 0, gxb = 0;
+        if constexpr (sizeof(R) == 8) {
+          oa[j] = ob[j] = R(0);
+          if (M::FULL || j < np) {
+            const double *v = saved + (6 * j) * kRevThreads + threadIdx.x;
+            const AngSaved A{v[0], v[kRevThreads], v[2 * kRevThreads]};
+            const AngSaved B{v[3 * kRevThreads], v[4 * kRevThreads], v[5 * kRevThreads]};
+            oa[j] = reverse_angle64(A, R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], dtv, r, gJx, ga);
+            ob[j] = reverse_angle64(B, R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], dtv, r, gJx, gb);
+            const R d = ga - gb;
+            lvx = fma(E.nx[j], d, lvx);
+            lvy = fma(E.ny[j], d, lvy);
+            lvz = fma(E.nz[j], d, lvz);
+          }
+          continue;
+        }
         oa[j] = reverse_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], E.ex(j, false, ci, k_ex),
                               dtv, r, gxa, ga);
         ob[j] = reverse_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex),
@@ -525,7 +596,13 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
 
 template <typename R, typename M> void launch_reverse_tile(rt_state *s, const AdjArgs<R> &a) {
   const unsigned g = (unsigned)((s->n_cells + kRevCells - 1) / kRevCells);
-  source_reverse_tile<R, M><<<g, kRevThreads, 0, s->stream>>>(a);
+  size_t sm = 0;
+  if constexpr (sizeof(R) == 8) {
+    sm = sizeof(double) * 6 * M::PPT * kRevThreads;  // 12 KB per pair, 98 KB at most
+    cudaFuncSetAttribute(source_reverse_tile<R, M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sm);
+  }
+  source_reverse_tile<R, M><<<g, kRevThreads, sm, s->stream>>>(a);
 }
 
 template <typename R, bool FULL> void reverse_pairs(rt_state *s, const AdjArgs<R> &a) {
