@@ -27,6 +27,7 @@
 
 #include "rt_internal.cuh"
 #include "rt_step_common.cuh"
+#include "rt_step_source.cuh"
 #include "rt_step_tile.cuh"
 
 namespace rt {
@@ -469,6 +470,7 @@ __global__ void __launch_bounds__(step::NT, M::PPT <= 6 ? 3 : 2)
   extern __shared__ __align__(128) unsigned char dyn[];
   const step::StageView v = step::stage_at(dyn, cap, false);
   step::issue_stage<false, false>(t, blockIdx.x, v);
+  if (threadIdx.x == 32) step::prefetch_ahead<false>(t, blockIdx.x);
   group_tile_body<float, M, true>(a, t, v);
 }
 
@@ -593,13 +595,15 @@ __device__ __forceinline__ void group_tile_body(const GroupArgs<R> &a, const Ste
     }
   } else {
     // float states (default): every lane finds the float root of the
-    // temperature equation from the float sums (no barrier); one lane per
-    // cell then refines it by a Newton step in double (the FP64 temperature
-    // solve) and forms the groups' q_j in float from it, or, where the float
-    // solve failed, runs the whole double chain.  Double states: the double
-    // chain, one lane per cell.
+    // temperature equation from the float sums and refines it
+    // (step::refine_quartic, no FP64).  Where a cell of the block needs more, the
+    // whole block goes on as double states do: one lane per cell refines the
+    // float root by a Newton step in double and forms the groups' q_j in float
+    // from it, or, where the float solve failed, runs the whole double chain.
+    // Double states: the double chain, one lane per cell.
     float Tf = 0.0f;
     unsigned fst = 1;
+    bool more = sizeof(R) == 8;
     if constexpr (sizeof(R) == 4) if (kind == RT_CELL_INTERIOR) {
       float4 kf[NG];
       load_kf(a, c, kf);
@@ -609,7 +613,11 @@ __device__ __forceinline__ void group_tile_body(const GroupArgs<R> &a, const Ste
           !quartic_root(k.alpha, rcv, k.gq, eint * rcp(rcv), 1e-7f, a.newton_max_iter, &Tf) &&
           isfinite(Tf))
         fst = 0;
+      float Tr;
+      more = fst != 0 || !step::refine_quartic(k.alpha, a.gs[c].rcv, rcv, k.gq, Tf, &Tr) ||
+             !group_q_f(a, kf, sI, sG, k, Tr, q);
     }
+    if (sizeof(R) == 8 || __syncthreads_or(more)) {
     if (sub == 0) {
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
@@ -663,6 +671,7 @@ __device__ __forceinline__ void group_tile_body(const GroupArgs<R> &a, const Ste
 #pragma unroll
     for (int g = 0; g < NG; ++g) q[g] = g < a.G ? sh.q[lc][g] : R(0);
     bad = sh.bad[lc];
+    }
   }
 
   // ---------------- phase C: new intensities and the radiation change
@@ -919,7 +928,10 @@ cudaError_t launch_fused_q(rt_state *s, double dt, const void *In, void *Out) {
   t.dt_r = (float)dt;
   const unsigned g = (unsigned)((s->n_cells + CPB - 1) / CPB);
   const int cap = step::stage_cap(s->max_block_slots);
-  group_step_fused<M><<<g, step::NT, step::stage_gas_offset(cap, false), s->stream>>>(a, t, cap);
+  const cudaError_t e = step::launch_carved(
+      group_step_fused<M>, g, step::NT, step::stage_gas_offset(cap, false), M::PPT <= 6 ? 3 : 2,
+      sizeof(TileShared<float>), false, s->stream, a, t, cap);
+  if (e != cudaSuccess) return e;
   s->launches++;
   return cudaGetLastError();
 }

@@ -109,6 +109,21 @@ __device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes) {
 // Tiles between a block's tile and the one it prefetches: a wave of four blocks
 // on each of 152 SMs.
 constexpr int kAhead = 608;
+// One thread of a block of tile `tile`: prefetch into L2 of the rows and slots of
+// the tile one wave of blocks ahead, so that the gathers and stages there find
+// them instead of waiting on HBM.
+template <bool MOVING>
+__device__ __forceinline__ void prefetch_ahead(const StepArgs<float> &a, int64_t tile) {
+  const int64_t c0 = (tile + kAhead) * CPB;
+  if (c0 >= a.n_cells) return;
+  const int64_t c1 = c0 + CPB < a.n_cells ? c0 + CPB : a.n_cells;
+  const int64_t k0 = a.ptr[c0], k1 = a.ptr[c1];
+  l2_prefetch(a.I_in + (size_t)c0 * a.row, (unsigned)(c1 - c0) * a.row * (unsigned)sizeof(float));
+  if (k1 > k0)
+    l2_prefetch((MOVING ? reinterpret_cast<const SlotF *>(a.slot) : a.slot_nb) + k0,
+                (unsigned)(k1 - k0) * (unsigned)sizeof(SlotF));
+}
+
 // Launches k with shared memory for `resident` blocks an SM (dynamic `sm` bytes
 // and `fixed` static ones each) and no more: the rest of the SM's 256 KB is L1
 // for the row gathers (the driver's split left them 121 KB: 2 % slower steps).
@@ -256,12 +271,14 @@ __device__ __forceinline__ void face_sum_quads(const SlotF *__restrict__ slot,
       const float2 D = pfma(NX[i], SX, pfma(NY[i], SY, pmul(NZ[i], SZ)));
       const float2 U = MOVING ? psub(D, W) : D;   // u of the two angles
       const float2 E = MOVING ? padd(D, W) : D;   // -u' of their antipodes
+      // min(u, 0) = u - max(u, 0) exactly
       const float2 UP = make_float2(fmaxf(U.x, 0.0f), fmaxf(U.y, 0.0f));
+      const float2 m1 = make_float2(-1.0f, -1.0f);
       const float2 EM = MOVING ? make_float2(fminf(E.x, 0.0f), fminf(E.y, 0.0f))
-                               : make_float2(fminf(U.x, 0.0f), fminf(U.y, 0.0f));
+                               : pfma(UP, m1, U);
       if constexpr (MODE == TRANSPORT_FORWARD) {
-        const float2 UM = MOVING ? make_float2(fminf(U.x, 0.0f), fminf(U.y, 0.0f)) : EM;
-        const float2 EP = MOVING ? make_float2(fmaxf(E.x, 0.0f), fmaxf(E.y, 0.0f)) : UP;
+        const float2 UM = MOVING ? pfma(UP, m1, U) : EM;
+        const float2 EP = MOVING ? pfma(EM, m1, E) : UP;
         CA[i] = pfma(UP, OA[i], pfma(UM, make_float2(v[i].x, v[i].y), CA[i]));
         CB[i] = pfma(EM, OB[i], pfma(EP, make_float2(v[i].z, v[i].w), CB[i]));
       } else {

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(NT, min_blocks<float, M::PPT>())
   extern __shared__ __align__(128) unsigned char dyn[];
   const StageView v = stage_at(dyn, cap, MOVING);
   issue_stage<MOVING, false>(a, blockIdx.x, v);
+  if (threadIdx.x == 32) prefetch_ahead<MOVING>(a, blockIdx.x);
   tile_transport<float, M, MOVING, true, MODE>(a, blockIdx.x, v);
 }
 
@@ -112,8 +113,11 @@ cudaError_t launch_tr(rt_state *s, double dt, const void *in, void *out) {
   const unsigned blocks = (unsigned)((s->n_cells + CPB - 1) / CPB);
   if constexpr (STAGED) {
     const int cap = stage_cap(s->max_block_slots);
-    transport_kernel_staged<M, MOVING, MODE>
-        <<<blocks, NT, stage_gas_offset(cap, MOVING), s->stream>>>(a, cap);
+    const cudaError_t e =
+        launch_carved(transport_kernel_staged<M, MOVING, MODE>, blocks, NT,
+                      stage_gas_offset(cap, MOVING), min_blocks<float, M::PPT>(), 0, false,
+                      s->stream, a, cap);
+    if (e != cudaSuccess) return e;
   } else {
     transport_kernel<R, M, MOVING, MODE><<<blocks, NT, 0, s->stream>>>(a);
   }
