@@ -621,6 +621,18 @@ int rt_create(const rt_mesh_desc *m_in, const rt_params *p, void *stream, rt_sta
     std::vector<int32_t> pos_of(angle_of.size());
     for (size_t q = 0; q < angle_of.size(); ++q) pos_of[(size_t)angle_of[q]] = (int32_t)q;
     CK(upload(s, &s->d_pos_of, pos_of));
+    // units of four positions: (x, x + 1, y, y + 1) in the quad region, (x, y, x + 1,
+    // y + 1) beyond it, x and y even (aligned to two values)
+    std::vector<int2> unit(A / 4);
+    bool ok = A % 4 == 0;
+    for (int u = 0; ok && u < A / 4; ++u) {
+      const int *c = &angle_of[4 * u];
+      const bool quad = 4 * u < s->quad_end;
+      const int x0 = c[0], x1 = quad ? c[1] : c[2], y0 = quad ? c[2] : c[1], y1 = c[3];
+      ok = x1 == x0 + 1 && y1 == y0 + 1 && x0 % 2 == 0 && y0 % 2 == 0;
+      unit[u] = make_int2(x0, y0);
+    }
+    if (ok) CK(upload(s, &s->d_unit_cols, unit));
   }
   CK(dalloc(s, &s->d_gs, N));
   CK(dalloc(s, &s->d_gd, N));
@@ -1401,7 +1413,7 @@ void rt_destroy(rt_state *s) {
     if (s->d_adj[k]) cudaFree(s->d_adj[k]);
   if (s->d_adj_ws) cudaFree(s->d_adj_ws);
   if (s->d_adj_stage) cudaFree(s->d_adj_stage);
-  void *bufs[] = {s->d_hface, s->d_hslot, s->d_hface_id, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_kout, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
+  void *bufs[] = {s->d_hface, s->d_hslot, s->d_hface_id, s->d_hlsq, s->d_hwork, s->d_kapgf, s->d_kapg, s->d_rkJ0, s->d_gcl_rate, s->d_gcl_kv, s->d_recon, s->d_lsq, s->d_Ihalf, s->d_grad, s->d_uface, s->d_kout, s->d_slot_nb, s->d_wface, s->d_angle_of, s->d_pos_of, s->d_unit_cols, s->d_cellv, s->d_ptr, s->d_nbr, s->d_slot, s->d_inv_vol, s->d_cell_of, s->d_volume, s->d_gs,
                   s->d_gd, s->d_kind, s->d_aux, s->d_bc_row, s->d_I0, s->d_ext, s->d_dir, s->d_wt,
                   s->d_dir64, s->d_wt64, s->d_qdir, s->d_mom, s->d_I[0], s->d_I[1], s->d_status, s->d_bad,
                   s->d_scratch, s->d_out16};

@@ -76,6 +76,79 @@ __global__ void permute_out_kernel(const R *__restrict__ src, R *__restrict__ ds
   }
 }
 
+// The same in units of four internal positions, for rows of a multiple of four
+// angles whose units hold the caller columns (x, x + 1) and (y, y + 1): one 16-byte
+// internal access (two of a double row) against two 8-byte caller accesses (16-byte),
+// neighbouring threads on neighbouring units, kUnits units in flight per thread.
+// 64^3 rows of 48 floats, in L2: 26 -> 16 us in, 22 -> 15 us out; bound by memory.
+constexpr int kUnits = 4;
+template <typename R> struct Two;
+template <> struct Two<float> { using t = float2; };
+template <> struct Two<double> { using t = double2; };
+__device__ __forceinline__ void load_unit(const float *p, float2 &x, float2 &y) {
+  const float4 v = *reinterpret_cast<const float4 *>(p);
+  x = make_float2(v.x, v.y);
+  y = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void load_unit(const double *p, double2 &x, double2 &y) {
+  x = reinterpret_cast<const double2 *>(p)[0];
+  y = reinterpret_cast<const double2 *>(p)[1];
+}
+__device__ __forceinline__ void store_unit(float *p, float2 x, float2 y) {
+  *reinterpret_cast<float4 *>(p) = make_float4(x.x, x.y, y.x, y.y);
+}
+__device__ __forceinline__ void store_unit(double *p, double2 x, double2 y) {
+  reinterpret_cast<double2 *>(p)[0] = x;
+  reinterpret_cast<double2 *>(p)[1] = y;
+}
+template <typename R, bool IN>
+__global__ void permute_units_kernel(const R *__restrict__ src, R *__restrict__ dst,
+                                     const int64_t *__restrict__ cell_of,
+                                     const int2 *__restrict__ unit_cols, int64_t n, int A,
+                                     int stride, int quad_end) {
+  using T = typename Two<R>::t;
+  const int U = A / 4;
+  const int64_t total = n * U, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < total;
+       i0 += kUnits * step) {
+    T x[kUnits], y[kUnits];
+    size_t in[kUnits], ox[kUnits], oy[kUnits];
+    bool quad[kUnits];
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) {
+      const int64_t i = i0 + k * step < total ? i0 + k * step : i0;
+      const int64_t row = total <= INT32_MAX ? (unsigned)i / (unsigned)U : i / U;
+      const int u = (int)(i - row * U);
+      const int2 c = unit_cols[u];
+      const size_t base = (size_t)cell_of[row] * A;
+      in[k] = (size_t)row * stride + 4 * u;
+      ox[k] = base + c.x;
+      oy[k] = base + c.y;
+      quad[k] = 4 * u < quad_end;
+      if (IN) {
+        x[k] = *reinterpret_cast<const T *>(src + ox[k]);
+        y[k] = *reinterpret_cast<const T *>(src + oy[k]);
+      } else {
+        load_unit(src + in[k], x[k], y[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kUnits; ++k) {
+      if (!quad[k]) {  // (x0, y0, x1, y1): the same exchange both ways
+        const R t = x[k].y;
+        x[k].y = y[k].x;
+        y[k].x = t;
+      }
+      if (IN) {
+        store_unit(dst + in[k], x[k], y[k]);
+      } else {
+        *reinterpret_cast<T *>(dst + ox[k]) = x[k];
+        *reinterpret_cast<T *>(dst + oy[k]) = y[k];
+      }
+    }
+  }
+}
+
 // Host-memory forms: lane k takes caller column k of the row (contiguous on
 // the host side) and the internal position pos_of[k].
 template <typename R>
@@ -399,29 +472,44 @@ unsigned permute_grid(int64_t n) {
 
 }  // namespace
 
+namespace {
+template <typename R, bool IN>
+void permute_rows(rt_state *s, const void *src, void *dst, int stride) {
+  const R *from = (const R *)src;
+  R *to = (R *)dst;
+  const int A = s->n_angles;
+  // units need the caller's rows aligned to their accesses (two values)
+  const uintptr_t caller = (uintptr_t)(IN ? src : dst);
+  if (s->d_unit_cols && stride % 4 == 0 && caller % (2 * sizeof(R)) == 0) {
+    const int64_t threads = (s->n_cells * (A / 4) + kUnits - 1) / kUnits;
+    const int64_t blocks = (threads + kThreads - 1) / kThreads;
+    permute_units_kernel<R, IN>
+        <<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), kThreads, 0, s->stream>>>(
+            from, to, s->d_cell_of, s->d_unit_cols, s->n_cells, A, stride, s->quad_end);
+  } else if (IN) {
+    permute_in_kernel<R><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
+        from, to, s->d_cell_of, s->d_angle_of, s->n_cells, A, stride);
+  } else {
+    permute_out_kernel<R><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
+        from, to, s->d_cell_of, s->d_angle_of, s->n_cells, A, stride);
+  }
+  s->launches++;
+}
+}  // namespace
+
 cudaError_t launch_permute_in(rt_state *s, const void *src, void *dst, int stride) {
   if (s->precision == RT_FP32)
-    permute_in_kernel<float><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
-        (const float *)src, (float *)dst, s->d_cell_of, s->d_angle_of, s->n_cells, s->n_angles,
-        stride);
+    permute_rows<float, true>(s, src, dst, stride);
   else
-    permute_in_kernel<double><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
-        (const double *)src, (double *)dst, s->d_cell_of, s->d_angle_of, s->n_cells,
-        s->n_angles, stride);
-  s->launches++;
+    permute_rows<double, true>(s, src, dst, stride);
   return cudaGetLastError();
 }
 
 cudaError_t launch_permute_out(rt_state *s, const void *src, void *dst, int stride) {
   if (s->precision == RT_FP32)
-    permute_out_kernel<float><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
-        (const float *)src, (float *)dst, s->d_cell_of, s->d_angle_of, s->n_cells, s->n_angles,
-        stride);
+    permute_rows<float, false>(s, src, dst, stride);
   else
-    permute_out_kernel<double><<<permute_grid(s->n_cells), kThreads, 0, s->stream>>>(
-        (const double *)src, (double *)dst, s->d_cell_of, s->d_angle_of, s->n_cells,
-        s->n_angles, stride);
-  s->launches++;
+    permute_rows<double, false>(s, src, dst, stride);
   return cudaGetLastError();
 }
 

@@ -247,6 +247,9 @@ struct rt_state {
   double *d_mom = nullptr;     // [A/2][kMomTab] moment coefficients of the pairs (rt_moments)
   int32_t *d_angle_of = nullptr;  // internal angle position -> caller angle
   int32_t *d_pos_of = nullptr;    // caller angle -> internal angle position
+  // [A/4] per unit of four internal positions the first caller columns of its two
+  // pairs of neighbouring columns (permute_units_kernel); NULL: no such units
+  int2 *d_unit_cols = nullptr;
   void *d_I[2] = {nullptr, nullptr};
   int cur = 0;
   unsigned *d_status = nullptr;
