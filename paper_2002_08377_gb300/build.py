@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librt_gb300.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["rt_api.cu", "rt_step.cu", "rt_step64.cu", "rt_transport.cu", "rt_aux.cu", "rt_adjoint.cu", "rt_noalloc.cu",
+SOURCES = ["rt_api.cu", "rt_step.cu", "rt_step64.cu", "rt_step_cell.cu", "rt_transport.cu", "rt_aux.cu", "rt_adjoint.cu", "rt_noalloc.cu",
            "rt_recon.cu", "rt_groups.cu", "rt_hydro.cu"]
 # per-file flags: the gas dynamics round as their plain formulas (no FMA contraction)
 FILE_FLAGS = {"rt_hydro.cu": ["--fmad=false"]}

@@ -574,6 +574,11 @@ int rt_create(const rt_mesh_desc *m_in, const rt_params *p, void *stream, rt_sta
     const cudaError_t e = upload(s, &s->d_qdir, qd);
     if (e != cudaSuccess) return bail(cuda_fail(s, e, "direction table"));
   }
+  for (int a = 0; a < A / 2 && A <= 8; ++a) {
+    for (int d = 0; d < 3; ++d) s->small_dir.push_back((float)m->angle_dir[3 * a + d]);
+    s->small_w.push_back((float)m->angle_w[a]);
+    s->small_w.push_back((float)m->angle_w[a + A / 2]);
+  }
   s->w_uni = m->angle_w[0];
   s->w_uniform = true;
   for (int a = 1; a < A; ++a) s->w_uniform = s->w_uniform && m->angle_w[a] == s->w_uni;

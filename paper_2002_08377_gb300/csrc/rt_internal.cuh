@@ -239,6 +239,7 @@ struct rt_state {
   void *d_cellv = nullptr;  // [N][4] in the state precision
   void *d_dir = nullptr;       // [A][4], caller angle order
   void *d_wt = nullptr;        // [A/2][2] weights of the pairs (p, p + A/2)
+  std::vector<float> small_dir, small_w;  // A <= 8: float directions [A/2][3], pair weights [A/2][2]
   bool w_uniform = false;      // every angle has the weight w_uni
   double w_uni = 0.0;
   float *d_qdir = nullptr;     // quad rows: the direction table of step::QuadDir
@@ -281,6 +282,9 @@ struct StepIO {
   bool src_only, commit;
 };
 cudaError_t launch_step_io(rt_state *s, double dt, const StepIO &io);
+// float states with at most 8 angles, two threads per cell (rt_step_cell.cu)
+bool cell_step_takes(const rt_state *s);
+cudaError_t launch_cell_step(rt_state *s, double dt, const StepIO &io);
 cudaError_t launch_step_io64(rt_state *s, double dt, const StepIO &io);  // double states (rt_step64.cu)
 // Transport only (rt_transport.cu), rows `in` -> `out` (stride row_stride):
 // adjoint = false: I* = I - dt/V sum_f u I_up; adjoint = true: the

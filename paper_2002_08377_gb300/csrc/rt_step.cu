@@ -696,6 +696,7 @@ template <bool MOVING> cudaError_t dispatch_quads(rt_state *s, double dt, const 
 cudaError_t dispatch(rt_state *s, double dt, const StepIO &io) {
   if (s->quad_end > 0)  // rows in the quad layout
     return s->moving ? dispatch_quads<true>(s, dt, io) : dispatch_quads<false>(s, dt, io);
+  if (cell_step_takes(s)) return launch_cell_step(s, dt, io);
   const bool full = (s->n_angles / 2) % KT == 0;
   if (s->moving)
     return full ? dispatch_pairs<true, true>(s, dt, io) : dispatch_pairs<true, false>(s, dt, io);
