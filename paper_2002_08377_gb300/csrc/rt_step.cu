@@ -302,15 +302,22 @@ struct QuadShared {
   unsigned bad[CPB];
 };
 
-// Resident threads per SM the register cap aims at.
-template <int NQ, bool TAIL, int T> constexpr int quad_blocks() {
-  return (2 * NQ + (TAIL ? 1 : 0) <= 5 ? 1024 : 768) / (CPB * T);
+// Resident threads per SM the register cap aims at; SMALL: meshes of at most two
+// blocks per SM (one wave at 128 registers), where the registers go into more loads
+// in flight.  Such a step is a chain of load latencies: us per step without / with
+// it 7.4 / 5.8 (16^3 cells x 48 angles), 9.0 / 6.8 (12^3 x 80), 18.8 / 11.1 (20^3 x
+// 128), 10.7 / 9.3 (16^3 x 96, moving); beyond one wave the halved residency costs
+// more than it gives.
+template <int NQ, bool TAIL, int T, bool SMALL> constexpr int quad_blocks() {
+  return (SMALL ? 512 : 2 * NQ + (TAIL ? 1 : 0) <= 5 ? 1024 : 768) / (CPB * T);
 }
+// Faces in flight per thread of a SMALL launch (what 128 registers hold).
+template <int NQ> constexpr int quad_chunk() { return NQ == 1 ? 8 : NQ == 2 ? 5 : 3; }
 
 // NQ quads and, with TAIL, one pair per thread; T threads per cell.  REFINE: the
 // float temperature root is refined (float_quartic = 0).
-template <int NQ, bool TAIL, int T, bool MOVING, bool REFINE>
-__global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
+template <int NQ, bool TAIL, int T, bool MOVING, bool REFINE, bool SMALL>
+__global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     quad_step_kernel(const __grid_constant__ StepArgs<float> a, const QuadDir qd, int cap) {
   constexpr int CW = 32 / T;  // cells per warp
   __shared__ QuadShared sh;
@@ -324,12 +331,15 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
   const int64_t c = live ? cell : a.n_cells - 1;  // dead lanes shadow the last cell
   const int RS = a.row;
 
-  // This kernel may start while the one before it in the stream runs its last
-  // blocks (programmatic dependent launch): what no kernel writes (slots, the
+  // A SMALL kernel may start while the one before it in the stream runs its last
+  // phase (programmatic dependent launch): what no kernel writes (slots, the
   // connectivity, kinds, directions) is loaded first, the wait comes before
-  // anything a kernel writes.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
+  // anything a kernel writes.  Blocks let the next kernel start once their rows are
+  // stored: at their start instead, the next kernel's blocks took slots and issue
+  // from this one's (16^3 cells x 48 angles 6.8 us per step, so 5.8, without 6.2).
+  // On larger meshes the same displacement costs more than the gap between kernels:
+  // 24^3 x 48 10.8 us with it, 9.8 without, 128^3 x 80 1132 and 1125 (32^3 x 80
+  // alone 24.2 and 25.0).
   // stage: each warp copies the slots and gas records of its own cells
   const int64_t kb = a.ptr[tile * CPB];
   const int64_t kc0 = a.ptr[c], kc1 = a.ptr[c + 1];
@@ -362,7 +372,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
     ty = d.y;
     tz = d.z;
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (SMALL) asm volatile("griddepcontrol.wait;" ::: "memory");
   {
     for (int i = lane; i < 6 * CW; i += 32) {
       const int cc = warp * CW + i / 6, k = i % 6;
@@ -414,7 +424,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
   }
   if (!a.src_only) {
     QuadSums<NQ> u;
-    quad_faces<NQ, TAIL, T, MOVING>(stage.slot, stage.nbr, (int)(kc0 - kb), (int)(kc1 - kb),
+    quad_faces<NQ, TAIL, T, MOVING, SMALL ? quad_chunk<NQ>() : 0>(stage.slot, stage.nbr, (int)(kc0 - kb), (int)(kc1 - kb),
                                     a.I_in, RS, sub, NX, NY, NZ, tx, ty, tz, IA, IB, IT, u);
     const float2 mdt = bcast(-dtv), pdt = bcast(dtv);
 #pragma unroll
@@ -617,6 +627,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
       dfz = fmaf(n.z, df, dfz);
     }
   }
+  if (SMALL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   {
     const float v[4] = {dea + deb, dfx, dfy, dfz};
     team_store4<T>(v, sub, lc, sh.sum);
@@ -634,23 +645,28 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T>())
   }
 }
 
-template <int NQ, bool TAIL, int T, bool MOVING>
-cudaError_t launch_quad(rt_state *s, double dt, const StepIO &io) {
-  const StepArgs<float> a = step_args<float>(s, dt, io);
-  const unsigned blocks = (unsigned)((s->n_cells + CPB - 1) / CPB);
+template <int NQ, bool TAIL, int T, bool MOVING, bool SMALL>
+cudaError_t launch_quad_as(rt_state *s, const StepArgs<float> &a, unsigned blocks) {
   const int cap = stage_cap(s->max_block_slots);
   const float4 *xy = reinterpret_cast<const float4 *>(s->d_qdir);
   const int Q = s->n_angles / 4;
   const QuadDir qd{xy, xy + Q, reinterpret_cast<const float2 *>(xy + 2 * Q)};
-  const size_t sm = stage_bytes(cap, MOVING);
-  auto *k = a.float_quartic ? quad_step_kernel<NQ, TAIL, T, MOVING, false>
-                            : quad_step_kernel<NQ, TAIL, T, MOVING, true>;
+  auto *k = a.float_quartic ? quad_step_kernel<NQ, TAIL, T, MOVING, false, SMALL>
+                            : quad_step_kernel<NQ, TAIL, T, MOVING, true, SMALL>;
   const cudaError_t e =
-      launch_carved(k, blocks, CPB * T, sm, quad_blocks<NQ, TAIL, T>(), sizeof(QuadShared), true,
-                    s->stream, a, qd, cap);
+      launch_carved(k, blocks, CPB * T, stage_bytes(cap, MOVING), quad_blocks<NQ, TAIL, T, SMALL>(),
+                    sizeof(QuadShared), SMALL, s->stream, a, qd, cap);
   if (e != cudaSuccess) return e;
   s->launches++;
   return cudaGetLastError();
+}
+
+template <int NQ, bool TAIL, int T, bool MOVING>
+cudaError_t launch_quad(rt_state *s, double dt, const StepIO &io) {
+  const StepArgs<float> a = step_args<float>(s, dt, io);
+  const unsigned blocks = (unsigned)((s->n_cells + CPB - 1) / CPB);
+  return blocks <= 2 * 152 ? launch_quad_as<NQ, TAIL, T, MOVING, true>(s, a, blocks)
+                           : launch_quad_as<NQ, TAIL, T, MOVING, false>(s, a, blocks);
 }
 
 template <typename M, bool MOVING>

@@ -60,7 +60,10 @@ template <int NQ> struct QuadSums {
 // the neighbour's, one of the two zero, so the pair of FMAs rounds as the
 // single product u I_up does.  min(u, 0) = u - max(u, 0) exactly.  (I_in is not
 // __restrict__: its loads must stay behind the wait for the kernel that wrote it.)
-template <int NQ, bool TAIL, int T, bool MOVING>
+// CHUNK > 0 (meshes that leave the SMs mostly idle): the rows of CHUNK faces are
+// loaded before the first one's arithmetic, the last chunk filled up with its
+// last face's loads.
+template <int NQ, bool TAIL, int T, bool MOVING, int CHUNK>
 __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr, int k0, int k1,
                                            const float *I_in, int RS, int sub,
                                            const float2 (&NX)[NQ], const float2 (&NY)[NQ],
@@ -71,22 +74,25 @@ __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr
 #pragma unroll
   for (int i = 0; i < NQ; ++i) o.CA[i] = o.CB[i] = bcast(0.0f);
   o.CT = bcast(0.0f);
-  constexpr int kUnroll = quad_unroll<NQ, TAIL, MOVING>();
-#pragma unroll kUnroll
-  for (int k = k0; k < k1; ++k) {
-    const float4 s = *reinterpret_cast<const float4 *>(slot + k);
-    const int nb = MOVING ? nbr[k] : __float_as_int(s.w);
+  struct Face {
+    float4 s, v[NQ];
+    float2 vt;
+  };
+  auto load = [&](int k, Face &f) {
+    f.s = *reinterpret_cast<const float4 *>(slot + k);
+    const int nb = MOVING ? nbr[k] : __float_as_int(f.s.w);
     const float *row = I_in + (size_t)nb * RS;
     const float4 *q = reinterpret_cast<const float4 *>(row) + sub;
-    float4 v[NQ];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) v[i] = q[T * i];
-    float2 vt = bcast(0.0f);
-    if (TAIL) vt = reinterpret_cast<const float2 *>(row)[2 * T * NQ + sub];
+    for (int i = 0; i < NQ; ++i) f.v[i] = q[T * i];
+    f.vt = TAIL ? reinterpret_cast<const float2 *>(row)[2 * T * NQ + sub] : bcast(0.0f);
+  };
+  auto add = [&](const Face &f) {
+    const float4 s = f.s;
     const float2 SX = bcast(s.x), SY = bcast(s.y), SZ = bcast(s.z);
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-      const float2 va = make_float2(v[i].x, v[i].y), vb = make_float2(v[i].z, v[i].w);
+      const float2 va = make_float2(f.v[i].x, f.v[i].y), vb = make_float2(f.v[i].z, f.v[i].w);
       const float2 D = pfma(NX[i], SX, pfma(NY[i], SY, pmul(NZ[i], SZ)));
       float2 U = D, E = D;  // u of the angles, -u of their antipodes
       if (MOVING) {
@@ -102,7 +108,25 @@ __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr
       const float d = fmaf(tx, s.x, fmaf(ty, s.y, tz * s.z));
       const float ua = MOVING ? d - s.w : d, ub = MOVING ? -d - s.w : -d;
       const bool pa = ua > 0.0f, pb = MOVING ? ub > 0.0f : !pa;
-      o.CT = pfma(make_float2(ua, ub), make_float2(pa ? OT.x : vt.x, pb ? OT.y : vt.y), o.CT);
+      o.CT = pfma(make_float2(ua, ub), make_float2(pa ? OT.x : f.vt.x, pb ? OT.y : f.vt.y), o.CT);
+    }
+  };
+  if constexpr (CHUNK > 0) {
+    for (int k = k0; k < k1; k += CHUNK) {
+      Face f[CHUNK];
+#pragma unroll
+      for (int j = 0; j < CHUNK; ++j) load(k + j < k1 ? k + j : k1 - 1, f[j]);
+#pragma unroll
+      for (int j = 0; j < CHUNK; ++j)
+        if (k + j < k1) add(f[j]);
+    }
+  } else {
+    constexpr int kUnroll = quad_unroll<NQ, TAIL, MOVING>();
+#pragma unroll kUnroll
+    for (int k = k0; k < k1; ++k) {
+      Face f;
+      load(k, f);
+      add(f);
     }
   }
 }
