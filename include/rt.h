@@ -100,8 +100,8 @@ typedef enum {
  *     too), rt_set_gas takes kappa_P, kappa_J, kappa_s as [N][n_groups], and
  *     rt_moments / rt_totals report the group-weighted sums.  Needs
  *     n_groups * A <= 128, RT_FIRST_ORDER, boost = 0, gcl = 0 and constant
- *     opacities; rt_adjoint_step refuses it.  A step is then two launches: the
- *     transport of all groups' intensities and the coupled source step. */
+ *     opacities; rt_adjoint_step refuses it.  A step transports all groups'
+ *     intensities and takes the coupled source step, in one launch or two. */
 typedef struct {
   int64_t n_cells;
   int64_t n_faces;
@@ -166,12 +166,13 @@ typedef enum { RT_FIRST_ORDER = 0, RT_VAN_LEER = 1 } rt_integrator;
  * graph of RT_GRAPH_STEPS steps captured on the state's stream (see rt_run);
  * 1 launches every kernel from the host.  Both give identical results.
  * float_quartic (RT_FP32 states only, ignored for RT_FP64): 0, the default,
- * solves the gas temperature equation of Eq. (com rad thermal disc) in
- * double -- its coefficients formed in double from the float angular sums,
- * Newton in double, one GPU lane per cell -- as the precision split of
- * RT_FP32 states says; 1 solves it in float in every lane of the cell (no
- * block barrier, faster; coefficients outside float range still take the
- * double solve), so the temperature carries float rounding.
+ * solves the gas temperature equation of Eq. (com rad thermal disc) to
+ * double accuracy, as the precision split of RT_FP32 states says: the emission
+ * it gives is the one that coefficients formed in double from the float angular
+ * sums and Newton in double give, rounded to float (found in float and refined
+ * by pairs of floats; where that is not certain, by the double Newton itself);
+ * 1 solves it in float alone (faster; coefficients outside float range still
+ * take the double solve), so the temperature carries float rounding.
  * hydro = 1 lets the state evolve the gas by the Euler equations as well
  * (rt_hydro_step, rt_radhydro_step: Sec. 2, radiation subcycled under a
  * hydro step); it needs face_offset, a static mesh (face_w NULL or zero),

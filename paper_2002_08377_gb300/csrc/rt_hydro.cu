@@ -29,7 +29,7 @@
 // what bounds the flux and gradient kernels: they are written for few FP64
 // instructions (FMAs, reciprocals of 3 FMAs, one side's star state only,
 // minima and maxima on the integer pipe).  64^3 linear-wave box, one van Leer
-// step: 3.2 -> 1.45 ms.  After the update the per-cell radiation coefficients
+// step: 3.2 -> 1.43 ms.  After the update the per-cell radiation coefficients
 // (rho kappa, rho c_v, 1 / rho) follow the new density (opacities per unit
 // mass are kept).
 #include <cuda_runtime.h>
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kThreads)
 //
 // One thread per cell and quantity, five neighbouring threads on a cell: a face's
 // five values are one run of 40 bytes to them.  (One thread per cell read each value
-// at a stride: 131 us at 64^3, five times what the additions take.)
+// at a stride: 131 us at 64^3, now 65; the additions alone take 35.)
 __global__ void update_kernel(const int64_t *__restrict__ ptr, const int32_t *__restrict__ face,
                               const double *__restrict__ flux, const double *__restrict__ vol,
                               int64_t n, double h, const GasStatic *__restrict__ gs_in,
