@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(step::NT, M::PPT <= 6 ? 3 : 2)
     group_step_fused(const GroupArgs<float> a, const StepArgs<float> t, int cap) {
   extern __shared__ __align__(128) unsigned char dyn[];
   const step::StageView v = step::stage_at(dyn, cap, false);
-  step::issue_stage<false, false>(t, blockIdx.x, v);
+  step::issue_stage<false>(t, blockIdx.x, v);
   if (threadIdx.x == 32) step::prefetch_ahead<false>(t, blockIdx.x);
   group_tile_body<float, M, true>(a, t, v);
 }

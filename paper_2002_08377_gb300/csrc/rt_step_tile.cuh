@@ -70,9 +70,9 @@ __device__ __forceinline__ StageView stage_at(unsigned char *base, int cap, bool
   return v;
 }
 
-// All threads: asynchronous copies of tile `tile`'s slots, neighbour indices
-// and (GAS) gas records into v (one contiguous range of each array).
-template <bool MOVING, bool GAS = true, int NTH = NT>
+// All threads: asynchronous copies of tile `tile`'s slots and neighbour indices
+// into v (one contiguous range of each array).
+template <bool MOVING>
 __device__ __forceinline__ void issue_stage(const StepArgs<float> &a, int64_t tile,
                                             const StageView &v) {
   const int64_t c0 = tile * CPB;
@@ -81,24 +81,12 @@ __device__ __forceinline__ void issue_stage(const StepArgs<float> &a, int64_t ti
   const int cnt = (int)(a.ptr[c1] - kb);
   if (MOVING) {
     const SlotF *gsl = reinterpret_cast<const SlotF *>(a.slot) + kb;
-    for (int i = threadIdx.x; i < cnt; i += NTH) {
+    for (int i = threadIdx.x; i < cnt; i += NT) {
       cp_async16(v.slot + i, gsl + i);
       cp_async4(v.nbr + i, a.nbr + kb + i);
     }
   } else {
-    for (int i = threadIdx.x; i < cnt; i += NTH) cp_async16(v.slot + i, a.slot_nb + kb + i);
-  }
-  if (!GAS) return;
-  // 6 x 16 bytes per cell: GasStatic (64) then GasDyn (32)
-  const int nc = (int)(c1 - c0);
-  for (int i = threadIdx.x; i < 6 * nc; i += NTH) {
-    const int cc = i / 6, k = i % 6;
-    if (k < 4)
-      cp_async16(reinterpret_cast<char *>(&v.gas->gs[cc]) + 16 * k,
-                 reinterpret_cast<const char *>(a.gs + c0 + cc) + 16 * k);
-    else
-      cp_async16(reinterpret_cast<char *>(&v.gas->gd[cc]) + 16 * (k - 4),
-                 reinterpret_cast<const char *>(a.gd + c0 + cc) + 16 * (k - 4));
+    for (int i = threadIdx.x; i < cnt; i += NT) cp_async16(v.slot + i, a.slot_nb + kb + i);
   }
 }
 

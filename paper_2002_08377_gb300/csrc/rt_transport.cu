@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(NT, min_blocks<float, M::PPT>())
     transport_kernel_staged(const StepArgs<float> a, int cap) {
   extern __shared__ __align__(128) unsigned char dyn[];
   const StageView v = stage_at(dyn, cap, MOVING);
-  issue_stage<MOVING, false>(a, blockIdx.x, v);
+  issue_stage<MOVING>(a, blockIdx.x, v);
   if (threadIdx.x == 32) prefetch_ahead<MOVING>(a, blockIdx.x);
   tile_transport<float, M, MOVING, true, MODE>(a, blockIdx.x, v);
 }
