@@ -194,8 +194,9 @@ __device__ __forceinline__ void gradient_chunk(const VLArgs<R> &a, int64_t c, in
 // it and the three-FMA face values 2.37 -> 1.97 ms).  The six operations of a face's
 // weight vector are done by one of the cell's eight threads, eight faces at a time,
 // and handed round by shuffles (a chunk has only two or four angles per thread to
-// share them): gradients of 41^3 x 48 1.06 -> 0.88 ms, the step 1.80.  The warp walks the faces together; past a cell's last face the
-// weights are zero and the last face's values come again, which changes nothing.
+// share them): gradients of 41^3 x 48 1.06 -> 0.88 ms, the step 1.80.  The warp
+// walks the faces together; past a cell's last face the weights are zero and the
+// last face's values come again, which changes nothing.
 // Every lane of the warp must call; live: c is the lane's own cell.
 template <typename M, int J0, int J1>
 __device__ __forceinline__ void gradient_chunk64(const VLArgs<double> &a, int64_t c, int sub,
