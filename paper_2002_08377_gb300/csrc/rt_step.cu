@@ -340,9 +340,13 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   // On larger meshes the same displacement costs more than the gap between kernels:
   // 24^3 x 48 10.8 us with it, 9.8 without, 128^3 x 80 1132 and 1125 (32^3 x 80
   // alone 24.2 and 25.0).
-  // stage: each warp copies the slots and gas records of its own cells
+  // stage: each warp copies the slots and gas records of its own cells and waits for
+  // nothing else, so it must not read what another warp copies: in a ragged last block
+  // every cell past the end gets its own copy of the last cell's record (below), and a
+  // warp that has only such cells takes no faces
   const int64_t kb = a.ptr[tile * CPB];
-  const int64_t kc0 = a.ptr[c], kc1 = a.ptr[c + 1];
+  const int64_t kc0 = a.ptr[c];
+  const int64_t kc1 = tile * CPB + warp * CW < a.n_cells ? a.ptr[c + 1] : kc0;
   {
     const int w0 = (int)(__shfl_sync(0xffffffffu, kc0, 0) - kb);
     const int w1 = (int)(__shfl_sync(0xffffffffu, kc1, 31) - kb);
@@ -376,15 +380,13 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   {
     for (int i = lane; i < 6 * CW; i += 32) {
       const int cc = warp * CW + i / 6, k = i % 6;
-      const int64_t gc = tile * CPB + cc;
-      if (gc < a.n_cells) {
-        if (k < 4)
-          cp_async16(reinterpret_cast<char *>(&stage.gas->gs[cc]) + 16 * k,
-                     reinterpret_cast<const char *>(a.gs + gc) + 16 * k);
-        else
-          cp_async16(reinterpret_cast<char *>(&stage.gas->gd[cc]) + 16 * (k - 4),
-                     reinterpret_cast<const char *>(a.gd + gc) + 16 * (k - 4));
-      }
+      const int64_t own = tile * CPB + cc, gc = own < a.n_cells ? own : a.n_cells - 1;
+      if (k < 4)
+        cp_async16(reinterpret_cast<char *>(&stage.gas->gs[cc]) + 16 * k,
+                   reinterpret_cast<const char *>(a.gs + gc) + 16 * k);
+      else
+        cp_async16(reinterpret_cast<char *>(&stage.gas->gd[cc]) + 16 * (k - 4),
+                   reinterpret_cast<const char *>(a.gd + gc) + 16 * (k - 4));
     }
   }
   // one warp prefetches the tile one wave of blocks ahead into L2, so that its
@@ -455,8 +457,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   // q / gamma^3; emitters: rate gamma, source / gamma^4).  A uniform weight cancels too.
   const float icr = a.inv_c_r;
   const float vx = cv.x * icr, vy = cv.y * icr, vz = cv.z * icr, eint = cv.w;
-  const int li = (int)(c - tile * CPB);
-  const GasStatic &gs = stage.gas->gs[li];
+  const GasStatic &gs = stage.gas->gs[lc];
   float xs = a.dt_cbar_r * (gs.frkJ + gs.frkS);
   double2 ax = make_double2(0.0, 0.0);
   if (kind != RT_CELL_INTERIOR) ax = a.aux[c];
@@ -548,7 +549,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     __syncthreads();  // before sh.sum and sh.bad are written again
   } else if (kind == RT_CELL_INTERIOR) {
     if (!source_q_fast<REFINE>(a, gs, sI, sG, s1, eint, q, bad)) {
-      const float2 r = source_q_slow(a, gs, stage.gas->gd[li], sI, sG, s1, eint);
+      const float2 r = source_q_slow(a, gs, stage.gas->gd[lc], sI, sG, s1, eint);
       q = r.x;
       bad |= __float_as_uint(r.y);
     }
