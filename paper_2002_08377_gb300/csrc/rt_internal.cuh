@@ -109,6 +109,8 @@ template <typename R> struct StepArgs {
   R dt_r, dt_cbar_r, inv_c_r;
   float k_dcr_f, k_alpha_f, k_g_f, a_rad_4pi_f;  // float copies for the float quartic
   int32_t newton_max_iter;
+  int32_t quick_iter;       // the refined float solve: its iteration limit and the relative
+  float quick_tol;          // change at which it stops (step::source_q_fast)
   int32_t float_quartic;    // float states: 1 solves the quartic in float in every lane
   int32_t src_only;         // 1: I_in holds I* already (no transport)
   int32_t commit;           // 0: the gas update is discarded (van Leer stage 1)

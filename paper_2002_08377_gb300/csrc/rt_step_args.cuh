@@ -167,6 +167,11 @@ template <typename R> StepArgs<R> step_args(rt_state *s, double dt, const StepIO
   a.k_fe = s->params.c / s->params.cbar * 4.0 * kPi;
   a.k_fm = 4.0 * kPi / s->params.cbar;
   a.newton_max_iter = s->params.newton_max_iter;
+  // iterations held back for the float solve to go on from a change of 1e-4 to 1e-7
+  constexpr int kSpare = 8;
+  const bool quick = a.newton_max_iter >= 2 * kSpare;
+  a.quick_iter = quick ? a.newton_max_iter - kSpare : a.newton_max_iter;
+  a.quick_tol = quick ? 1e-4f : 1e-7f;
   a.float_quartic = s->params.float_quartic;
   a.k_dcr_f = (float)a.k_dcr;
   a.k_alpha_f = (float)a.k_alpha;

@@ -118,7 +118,11 @@ static __device__ __noinline__ float2 source_q_slow(const StepArgs<float> &a, co
 // with float_quartic = 1 (REFINE false) as it is.  The refined Newton stops at a
 // relative change of 1e-4: it converges quadratically (e -> 1.5 e^2 at most), so
 // the root is then within float rounding and the refinement squares what is
-// left.  Returns false where source_q_slow has to take over.
+// left.  Going on to 1e-7, where source_q_slow's float Newton stops, takes at most
+// two more iterations (1e8 random equations, quotients off by up to 2 ulp); so that
+// newton_max_iter refuses the same cells as if it went on, the early stop counts
+// only 8 iterations before the limit (StepArgs::quick_iter), and a limit below 16
+// stops at 1e-7.  Returns false where source_q_slow has to take over.
 template <bool REFINE>
 __device__ __forceinline__ bool source_q_fast(const StepArgs<float> &a, const GasStatic &gr,
                                               float SI, float SG, float S1, float eint,
@@ -132,7 +136,7 @@ __device__ __forceinline__ bool source_q_fast(const StepArgs<float> &a, const Ga
   if (REFINE) {
     float Tf;
     if (a.beta_P_f != 0.0f || !isfinite(k.alpha) || !isfinite(k.gq) ||
-        quartic_root(k.alpha, gr.frcv, k.gq, eint * rcp(gr.frcv), 1e-4f, a.newton_max_iter, &Tf) ||
+        quartic_root(k.alpha, gr.frcv, k.gq, eint * rcp(gr.frcv), a.quick_tol, a.quick_iter, &Tf) ||
         !refine_quartic(k.alpha, gr.rcv, gr.frcv, k.gq, Tf, &T))
       return false;
     q = float_q(a, k, T, SI, SG);
