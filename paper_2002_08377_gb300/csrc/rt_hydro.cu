@@ -49,6 +49,7 @@ constexpr int kThreads = 256;
 
 using step::key_value;
 using step::order_key;
+using step::quotient;
 using step::rcp;
 
 // primitive (rho, vx, vy, vz, P) of a conserved state
@@ -305,8 +306,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     // Barth-Jespersen: the largest factor keeping every face value in [lo, hi]
     const double up = key_value(dmax[q]), dn = key_value(dmin[q]);
     double alpha = 1.0;
-    if (up > 0.0) alpha = fmin(alpha, (key_value(hi[q]) - v[q]) * rcp(up));
-    if (dn < 0.0) alpha = fmin(alpha, (key_value(lo[q]) - v[q]) * rcp(dn));
+    if (up > 0.0) alpha = fmin(alpha, quotient(key_value(hi[q]) - v[q], up));
+    if (dn < 0.0) alpha = fmin(alpha, quotient(key_value(lo[q]) - v[q], dn));
 #pragma unroll
     for (int x = 0; x < 3; ++x) out[5 * x + q] = g[q][x] * alpha;
   }

@@ -270,8 +270,8 @@ __device__ __forceinline__ void gradient_chunk64(const VLArgs<double> &a, int64_
   for (int u = 0; u < 2 * J; ++u) {
     const double x = key_value(up[u]), n = key_value(dn[u]);
     double f = 1.0;
-    if (x > 0.0) f = fmin(f, (key_value(hi[u]) - v[u]) * rcp(x));
-    if (n < 0.0) f = fmin(f, (key_value(lo[u]) - v[u]) * rcp(n));
+    if (x > 0.0) f = fmin(f, quotient(key_value(hi[u]) - v[u], x));
+    if (n < 0.0) f = fmin(f, quotient(key_value(lo[u]) - v[u], n));
 #pragma unroll
     for (int d = 0; d < 3; ++d) (u & 1 ? gb : ga)[d][J0 + u / 2] = b[u][d] * f;
   }

@@ -45,7 +45,7 @@ __device__ __forceinline__ double source_q(const StepArgs<R> &a, const GasStatic
   if (!(gq >= 0.0) || !(alpha >= 0.0)) {
     bad |= ST_NONFINITE;
   } else if (a.beta_P == 0.0) {
-    if (quartic_root(alpha, g.rcv, gq, eint * rcp(g.rcv), 1e-15, a.newton_max_iter, &T))
+    if (quartic_root(alpha, g.rcv, gq, quotient(eint, g.rcv), 1e-15, a.newton_max_iter, &T))
       bad |= ST_NONCONV;
   } else {
     // kappa_P (T/T_ref)^beta_P T^4 = kappa_P T_ref^-beta_P T^(4 + beta_P)

@@ -54,15 +54,22 @@ __device__ __forceinline__ float rcp(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-__device__ __forceinline__ double rcp(double x) {
+__device__ __forceinline__ bool rcp_range(double x) {
   // |x| in [2^-1000, 2^1001) <=> biased exponent in [23, 2024), tested on the
   // integer pipe (the FP64 pipe is the double kernels' bottleneck)
-  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-  if (ex - 23u >= 2001u) return 1.0 / x;
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 23u < 2001u;
+}
+__device__ __forceinline__ double rcp(double x) {
+  if (!rcp_range(x)) return 1.0 / x;
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
+}
+// a / b within 2 ulp.  Where 1 / b could leave the range of a double (b subnormal: the
+// reciprocal is infinite and 0 times it no number) the IEEE division.
+__device__ __forceinline__ double quotient(double a, double b) {
+  return rcp_range(b) ? a * rcp(b) : a / b;
 }
 template <typename R> __device__ __forceinline__ pair_t<R> prcp(pair_t<R> v) {
   return mk(rcp(v.x), rcp(v.y));
@@ -160,7 +167,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // bound g / beta.  The iteration stops when an iterate fails to decrease or
 // moves by at most `tol` of itself.  Returns 1 if it did not converge.
 __device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double qdiv(double a, double b) { return a * rcp(b); }
+__device__ __forceinline__ double qdiv(double a, double b) { return quotient(a, b); }
 
 template <typename T_>
 __device__ __forceinline__ int quartic_root(T_ alpha, T_ beta, T_ g, T_ T0, T_ tol, int max_iter,
