@@ -314,6 +314,14 @@ template <int NQ, bool TAIL, int T, bool SMALL> constexpr int quad_blocks() {
 // Faces in flight per thread of a SMALL launch (what 128 registers hold).
 template <int NQ> constexpr int quad_chunk() { return NQ == 1 ? 8 : NQ == 2 ? 5 : 3; }
 
+// The warp that does a block's lane-per-cell double work. It rotates with the block, so
+// that the SM's four schedulers share that work; in a ragged last block it is one that
+// has cells.
+template <int T> __device__ __forceinline__ int cell_warp(int64_t tile, int64_t n_cells) {
+  const int w = (int)(tile % T);
+  return tile * CPB + w * (32 / T) < n_cells ? w : 0;
+}
+
 // NQ quads and, with TAIL, one pair per thread; T threads per cell.  REFINE: the
 // float temperature root is refined (float_quartic = 0).
 template <int NQ, bool TAIL, int T, bool MOVING, bool REFINE, bool SMALL>
@@ -341,16 +349,17 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   // 24^3 x 48 10.8 us with it, 9.8 without, 128^3 x 80 1132 and 1125 (32^3 x 80
   // alone 24.2 and 25.0).
   // stage: each warp copies the slots and gas records of its own cells and waits for
-  // nothing else, so it must not read what another warp copies: in a ragged last block
-  // every cell past the end gets its own copy of the last cell's record (below), and a
-  // warp that has only such cells takes no faces
+  // nothing else, so it must not read what another warp copies.  A warp of the last
+  // block whose cells all lie past the end (its lanes would take the last cell's
+  // record) copies nothing and leaves below; block barriers wait for the threads that
+  // have not left.
+  const bool alive = tile * CPB + warp * CW < a.n_cells;
   const int64_t kb = a.ptr[tile * CPB];
-  const int64_t kc0 = a.ptr[c];
-  const int64_t kc1 = tile * CPB + warp * CW < a.n_cells ? a.ptr[c + 1] : kc0;
+  const int64_t kc0 = a.ptr[c], kc1 = a.ptr[c + 1];
   {
     const int w0 = (int)(__shfl_sync(0xffffffffu, kc0, 0) - kb);
     const int w1 = (int)(__shfl_sync(0xffffffffu, kc1, 31) - kb);
-    if (!a.src_only) {
+    if (alive && !a.src_only) {
       const SlotF *g = (MOVING ? reinterpret_cast<const SlotF *>(a.slot) : a.slot_nb) + kb;
       for (int i = w0 + lane; i < w1; i += 32) {
         cp_async16(stage.slot + i, g + i);
@@ -376,17 +385,20 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     ty = d.y;
     tz = d.z;
   }
+  if (!alive) return;  // (at the top of the kernel it costs registers: 64^3 x 48 3 % longer)
   if (SMALL) asm volatile("griddepcontrol.wait;" ::: "memory");
   {
     for (int i = lane; i < 6 * CW; i += 32) {
       const int cc = warp * CW + i / 6, k = i % 6;
-      const int64_t own = tile * CPB + cc, gc = own < a.n_cells ? own : a.n_cells - 1;
-      if (k < 4)
-        cp_async16(reinterpret_cast<char *>(&stage.gas->gs[cc]) + 16 * k,
-                   reinterpret_cast<const char *>(a.gs + gc) + 16 * k);
-      else
-        cp_async16(reinterpret_cast<char *>(&stage.gas->gd[cc]) + 16 * (k - 4),
-                   reinterpret_cast<const char *>(a.gd + gc) + 16 * (k - 4));
+      const int64_t gc = tile * CPB + cc;
+      if (gc < a.n_cells) {
+        if (k < 4)
+          cp_async16(reinterpret_cast<char *>(&stage.gas->gs[cc]) + 16 * k,
+                     reinterpret_cast<const char *>(a.gs + gc) + 16 * k);
+        else
+          cp_async16(reinterpret_cast<char *>(&stage.gas->gd[cc]) + 16 * (k - 4),
+                     reinterpret_cast<const char *>(a.gd + gc) + 16 * (k - 4));
+      }
     }
   }
   // one warp prefetches the tile one wave of blocks ahead into L2, so that its
@@ -457,7 +469,8 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   // q / gamma^3; emitters: rate gamma, source / gamma^4).  A uniform weight cancels too.
   const float icr = a.inv_c_r;
   const float vx = cv.x * icr, vy = cv.y * icr, vz = cv.z * icr, eint = cv.w;
-  const GasStatic &gs = stage.gas->gs[lc];
+  const int li = (int)(c - tile * CPB);
+  const GasStatic &gs = stage.gas->gs[li];
   float xs = a.dt_cbar_r * (gs.frkJ + gs.frkS);
   double2 ax = make_double2(0.0, 0.0);
   if (kind != RT_CELL_INTERIOR) ax = a.aux[c];
@@ -527,7 +540,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     }
     __syncthreads();
     const int64_t cl = tile * CPB + lane;
-    if (warp == (int)(tile % T) && cl < a.n_cells) {
+    if (warp == cell_warp<T>(tile, a.n_cells) && cl < a.n_cells) {
       float2 r = bcast(0.0f);
       if (a.kind[cl] == RT_CELL_INTERIOR) {
         float ql = 0.0f;
@@ -549,7 +562,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     __syncthreads();  // before sh.sum and sh.bad are written again
   } else if (kind == RT_CELL_INTERIOR) {
     if (!source_q_fast<REFINE>(a, gs, sI, sG, s1, eint, q, bad)) {
-      const float2 r = source_q_slow(a, gs, stage.gas->gd[lc], sI, sG, s1, eint);
+      const float2 r = source_q_slow(a, gs, stage.gas->gd[li], sI, sG, s1, eint);
       q = r.x;
       bad |= __float_as_uint(r.y);
     }
@@ -638,7 +651,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
 
   // ---------------- phase D: gas exchange, one lane per cell
   const int64_t cl = tile * CPB + lane;
-  if (warp == (int)(tile % T) && cl < a.n_cells) {
+  if (warp == cell_warp<T>(tile, a.n_cells) && cl < a.n_cells) {
     unsigned b = sh.bad[lane];
     if (!isfinite(sh.sum[0][lane])) b |= ST_NONFINITE;
     gas_exchange<float, MOVING>(a, cl, stage.gas->gs[lane], stage.gas->gd[lane], sh.sum[0][lane],
