@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(NT, min_blocks<M::PPT>()) step_kernel(const St
     // are already in all 8 lanes), no block barrier
     if (kind == RT_CELL_INTERIOR)
       if (!source_q_fast<false>(a, a.gs[c], sI, sG, s1, eint, q, bad)) {
-        const float2 r = source_q_slow(a, a.gs[c], a.gd[c], sI, sG, s1, eint);
+        const float2 r = source_q_double(a, a.gs[c], a.gd[c], sI, sG, s1, eint);
         q = r.x;
         bad |= __float_as_uint(r.y);
       }
@@ -562,7 +562,9 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     __syncthreads();  // before sh.sum and sh.bad are written again
   } else if (kind == RT_CELL_INTERIOR) {
     if (!source_q_fast<REFINE>(a, gs, sI, sG, s1, eint, q, bad)) {
-      const float2 r = source_q_slow(a, gs, stage.gas->gd[li], sI, sG, s1, eint);
+      const GasDyn &gd = stage.gas->gd[li];
+      const float2 r = REFINE || NQ > 2 ? source_q_slow(a, gs, gd, sI, sG, s1, eint)
+                                        : source_q_double(a, gs, gd, sI, sG, s1, eint);
       q = r.x;
       bad |= __float_as_uint(r.y);
     }

@@ -94,11 +94,10 @@ __device__ __forceinline__ float float_q(const StepArgs<float> &a, const Quartic
 // source_q_fast could not give: power-law opacities and values out of range of
 // refine_quartic take the float root refined in double by refine_root; where a
 // float value is not finite or the float Newton did not converge, the double
-// solve of source_q.  Returns q and the status bits.  Out of line: rare, and its
-// registers are many.
-static __device__ __noinline__ float2 source_q_slow(const StepArgs<float> &a, const GasStatic &gr,
-                                             const GasDyn &gd, float SI, float SG, float S1,
-                                             float eint) {
+// solve of source_q.  Returns q and the status bits.
+__device__ __forceinline__ float2 source_q_double(const StepArgs<float> &a, const GasStatic &gr,
+                                                  const GasDyn &gd, float SI, float SG, float S1,
+                                                  float eint) {
   const QuarticF k = float_coeffs(a, gr.frkP, gr.frkJ, gr.frkS, eint, SI, SG, S1);
   float Tf;
   if (isfinite(k.alpha) && isfinite(k.gq) && !float_root(a, k, gr.frcv, eint, &Tf) &&
@@ -110,6 +109,20 @@ static __device__ __noinline__ float2 source_q_slow(const StepArgs<float> &a, co
   unsigned bad = 0;
   const double q = source_q(a, gr, gd, (double)SI, (double)SG, (double)S1, bad);
   return make_float2((float)q, __uint_as_float(bad));
+}
+
+// The same out of line, for the kernels that refine in every lane of the cell: rare
+// there, and its registers are many.  Where it is all of the float path (float_quartic
+// = 1) or one lane per cell runs it (step_kernel), the call costs more than it saves:
+// the registers that the ABI keeps across it spill in the loops around.  us per step
+// with the call and without, 56^3 cells: 104 angles 354 and 248, 72 angles 173 and
+// 154, float_quartic = 1 with 24 angles 98 and 97 (32^3 x 104: 72 and 47); quad rows
+// with float_quartic = 1, 48^3 x 48: 57.4 and 55.2 (three quads a thread and more keep
+// the call: 64^3 x 112 222 with it and 267 without).
+static __device__ __noinline__ float2 source_q_slow(const StepArgs<float> &a, const GasStatic &gr,
+                                                    const GasDyn &gd, float SI, float SG, float S1,
+                                                    float eint) {
+  return source_q_double(a, gr, gd, SI, SG, S1, eint);
 }
 
 // q of an interior cell in float, in every lane of the cell, from the float
@@ -159,7 +172,7 @@ __device__ __forceinline__ float source_q_refined(const StepArgs<float> &a, cons
                                                   float eint, unsigned &bad) {
   float q = 0.0f;
   if (source_q_fast<true>(a, gr, SI, SG, S1, eint, q, bad)) return q;
-  const float2 r = source_q_slow(a, gr, gd, SI, SG, S1, eint);
+  const float2 r = source_q_double(a, gr, gd, SI, SG, S1, eint);
   bad |= __float_as_uint(r.y);
   return r.x;
 }
