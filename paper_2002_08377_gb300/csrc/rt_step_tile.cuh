@@ -259,11 +259,14 @@ __device__ __forceinline__ void face_sum_quads(const SlotF *__restrict__ slot,
       const float2 D = pfma(NX[i], SX, pfma(NY[i], SY, pmul(NZ[i], SZ)));
       const float2 U = MOVING ? psub(D, W) : D;   // u of the two angles
       const float2 E = MOVING ? padd(D, W) : D;   // -u' of their antipodes
-      // min(u, 0) = u - max(u, 0) exactly
+      // min(u, 0) = u - max(u, 0) exactly; the transposed sweep with four quads a thread
+      // takes the minimum itself (the difference spills there: reverse step of 64^3 x 128
+      // 888 us with the minimum, 932 with the difference, 913 before it)
+      constexpr bool kDiff = Q4 < 4 || MODE == TRANSPORT_FORWARD;
       const float2 UP = make_float2(fmaxf(U.x, 0.0f), fmaxf(U.y, 0.0f));
       const float2 m1 = make_float2(-1.0f, -1.0f);
-      const float2 EM = MOVING ? make_float2(fminf(E.x, 0.0f), fminf(E.y, 0.0f))
-                               : pfma(UP, m1, U);
+      const float2 EM = MOVING || !kDiff ? make_float2(fminf(E.x, 0.0f), fminf(E.y, 0.0f))
+                                         : pfma(UP, m1, U);
       if constexpr (MODE == TRANSPORT_FORWARD) {
         const float2 UM = MOVING ? pfma(UP, m1, U) : EM;
         const float2 EP = MOVING ? pfma(EM, m1, E) : UP;
