@@ -490,12 +490,12 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
             v[3 * kRevThreads] = B.iG;
             v[4 * kRevThreads] = B.r;
             v[5 * kRevThreads] = B.ex;
-            continue;
+          } else {
+            sums_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], E.ex(j, false, ci, k_ex), Nw,
+                       SI, SG, S1, lq);
+            sums_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex), Nw, SI,
+                       SG, S1, lq);
           }
-          sums_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], E.ex(j, false, ci, k_ex), Nw, SI,
-                     SG, S1, lq);
-          sums_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex), Nw, SI,
-                     SG, S1, lq);
         }
     }
     cs = CellSums<R>{group_sum(Nw), group_sum(SI), group_sum(SG), group_sum(S1), group_sum(lq)};
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
 #pragma unroll
       for (int j = 0; j < PPT; ++j) {
         const R t = fma(ci.bx, E.nx[j], fma(ci.by, E.ny[j], ci.bz * E.nz[j]));
-        R ga = 0, gb = 0, gxa = 0, gxb = 0;
+        R ga = 0, gb = 0;
         if constexpr (sizeof(R) == 8) {
           oa[j] = ob[j] = R(0);
           if (M::FULL || j < np) {
@@ -563,18 +563,19 @@ __global__ void __launch_bounds__(kRevThreads, sizeof(R) == 4 ? (M::PPT <= 5 ? 4
             lvy = fma(E.ny[j], d, lvy);
             lvz = fma(E.nz[j], d, lvz);
           }
-          continue;
-        }
-        oa[j] = reverse_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j], E.ex(j, false, ci, k_ex),
-                              dtv, r, gxa, ga);
-        ob[j] = reverse_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex),
-                              dtv, r, gxb, gb);
-        if (M::FULL || j < np) {
-          gJx += gxa + gxb;
-          const R d = ga - gb;
-          lvx = fma(E.nx[j], d, lvx);
-          lvy = fma(E.ny[j], d, lvy);
-          lvz = fma(E.nz[j], d, lvz);
+        } else {
+          R gxa = 0, gxb = 0;
+          oa[j] = reverse_angle(R(1) - t, E.wa[j], ci.X, E.Ia[j], E.la[j],
+                                E.ex(j, false, ci, k_ex), dtv, r, gxa, ga);
+          ob[j] = reverse_angle(R(1) + t, E.wb[j], ci.X, E.Ib[j], E.lb[j], E.ex(j, true, ci, k_ex),
+                                dtv, r, gxb, gb);
+          if (M::FULL || j < np) {
+            gJx += gxa + gxb;
+            const R d = ga - gb;
+            lvx = fma(E.nx[j], d, lvx);
+            lvy = fma(E.ny[j], d, lvy);
+            lvz = fma(E.nz[j], d, lvz);
+          }
         }
       }
     }

@@ -308,8 +308,8 @@ struct QuadShared {
 // it 7.4 / 5.8 (16^3 cells x 48 angles), 9.0 / 6.8 (12^3 x 80), 18.8 / 11.1 (20^3 x
 // 128), 10.7 / 9.3 (16^3 x 96, moving); beyond one wave the halved residency costs
 // more than it gives.
-template <int NQ, bool TAIL, int T, bool SMALL> constexpr int quad_blocks() {
-  return (SMALL ? 512 : 2 * NQ + (TAIL ? 1 : 0) <= 5 ? 1024 : 768) / (CPB * T);
+template <int NQ, bool TAIL, bool SMALL> constexpr int quad_blocks() {
+  return (SMALL ? 512 : 2 * NQ + (TAIL ? 1 : 0) <= 5 ? 1024 : 768) / NT;
 }
 // Faces in flight per thread of a SMALL launch (what 128 registers hold).
 template <int NQ> constexpr int quad_chunk() { return NQ == 1 ? 8 : NQ == 2 ? 5 : 3; }
@@ -317,23 +317,23 @@ template <int NQ> constexpr int quad_chunk() { return NQ == 1 ? 8 : NQ == 2 ? 5 
 // The warp that does a block's lane-per-cell double work. It rotates with the block, so
 // that the SM's four schedulers share that work; in a ragged last block it is one that
 // has cells.
-template <int T> __device__ __forceinline__ int cell_warp(int64_t tile, int64_t n_cells) {
-  const int w = (int)(tile % T);
-  return tile * CPB + w * (32 / T) < n_cells ? w : 0;
+__device__ __forceinline__ int cell_warp(int64_t tile, int64_t n_cells) {
+  const int w = (int)(tile % KT);
+  return tile * CPB + w * (32 / KT) < n_cells ? w : 0;
 }
 
-// NQ quads and, with TAIL, one pair per thread; T threads per cell.  REFINE: the
+// NQ quads and, with TAIL, one pair per thread; KT threads per cell.  REFINE: the
 // float temperature root is refined (float_quartic = 0).
-template <int NQ, bool TAIL, int T, bool MOVING, bool REFINE, bool SMALL>
-__global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
+template <int NQ, bool TAIL, bool MOVING, bool REFINE, bool SMALL>
+__global__ void __launch_bounds__(NT, quad_blocks<NQ, TAIL, SMALL>())
     quad_step_kernel(const __grid_constant__ StepArgs<float> a, const QuadDir qd, int cap) {
-  constexpr int CW = 32 / T;  // cells per warp
+  constexpr int CW = 32 / KT;  // cells per warp
   __shared__ QuadShared sh;
   extern __shared__ __align__(128) unsigned char dyn[];
   const int64_t tile = blockIdx.x;
   const StageView stage = stage_at(dyn, cap, MOVING);
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int lc = threadIdx.x / T, sub = threadIdx.x % T;
+  const int lc = threadIdx.x / KT, sub = threadIdx.x % KT;
   const int64_t cell = tile * CPB + lc;
   const bool live = cell < a.n_cells;
   const int64_t c = live ? cell : a.n_cells - 1;  // dead lanes shadow the last cell
@@ -371,13 +371,13 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   float2 NX[NQ], NY[NQ], NZ[NQ];
 #pragma unroll
   for (int i = 0; i < NQ; ++i) {
-    const float4 d = __ldg(qd.xy + sub + T * i);
-    const float2 z = __ldg(reinterpret_cast<const float2 *>(qd.zw + sub + T * i));
+    const float4 d = __ldg(qd.xy + sub + KT * i);
+    const float2 z = __ldg(reinterpret_cast<const float2 *>(qd.zw + sub + KT * i));
     NX[i] = make_float2(d.x, d.y);
     NY[i] = make_float2(d.z, d.w);
     NZ[i] = z;
   }
-  const float4 *tdir = reinterpret_cast<const float4 *>(a.dir) + 2 * T * NQ + sub;
+  const float4 *tdir = reinterpret_cast<const float4 *>(a.dir) + 2 * KT * NQ + sub;
   float tx = 0.0f, ty = 0.0f, tz = 0.0f;
   if (TAIL) {
     const float4 d = __ldg(tdir);
@@ -430,16 +430,17 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     const float *o = a.I_in + (size_t)c * RS;
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-      const float4 t = reinterpret_cast<const float4 *>(o)[sub + T * i];
+      const float4 t = reinterpret_cast<const float4 *>(o)[sub + KT * i];
       IA[i] = make_float2(t.x, t.y);
       IB[i] = make_float2(t.z, t.w);
     }
-    if (TAIL) IT = reinterpret_cast<const float2 *>(o)[2 * T * NQ + sub];
+    if (TAIL) IT = reinterpret_cast<const float2 *>(o)[2 * KT * NQ + sub];
   }
   if (!a.src_only) {
     QuadSums<NQ> u;
-    quad_faces<NQ, TAIL, T, MOVING, SMALL ? quad_chunk<NQ>() : 0>(stage.slot, stage.nbr, (int)(kc0 - kb), (int)(kc1 - kb),
-                                    a.I_in, RS, sub, NX, NY, NZ, tx, ty, tz, IA, IB, IT, u);
+    quad_faces<NQ, TAIL, MOVING, SMALL ? quad_chunk<NQ>() : 0>(
+        stage.slot, stage.nbr, (int)(kc0 - kb), (int)(kc1 - kb), a.I_in, RS, sub, NX, NY, NZ, tx,
+        ty, tz, IA, IB, IT, u);
     const float2 mdt = bcast(-dtv), pdt = bcast(dtv);
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
@@ -478,7 +479,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   const float gam = frame_gamma(a.boost, vx, vy, vz);
   if (a.boost) xs *= gam;
   const bool uw = a.w_uniform;
-  const float2 *W2 = reinterpret_cast<const float2 *>(a.wt2) + 2 * T * NQ + sub;  // the tail pair's
+  const float2 *W2 = reinterpret_cast<const float2 *>(a.wt2) + 2 * KT * NQ + sub;  // the tail pair's
   // the sums over a thread's angles run over its pairs in order, the first
   // angles' (x) and the antipodes' (y) apart
   float2 sIv = bcast(0.0f), sGv = sIv, s1v = sIv;
@@ -494,9 +495,9 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
       float2 ta = prcpf(pmul(GA2, pfma(XS, GA, one))), tb = prcpf(pmul(GB2, pfma(XS, GB, one)));
       float2 wa = bcast(a.w_uni), wb = wa;
       if (!uw) {
-        const float4 d = __ldg(qd.zw + sub + T * i);
+        const float4 d = __ldg(qd.zw + sub + KT * i);
         wa = make_float2(d.z, d.w);
-        wb = __ldg(qd.wb + sub + T * i);
+        wb = __ldg(qd.wb + sub + KT * i);
       }
       ta = pmul(wa, ta);
       tb = pmul(wb, tb);
@@ -518,8 +519,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
       sGv = pfma(t, G, sGv);
     }
   }
-  float sI = team_sum<T>(sIv.x + sIv.y), sG = team_sum<T>(sGv.x + sGv.y),
-        s1 = team_sum<T>(s1v.x + s1v.y);
+  float sI = cell_sum(sIv.x + sIv.y), sG = cell_sum(sGv.x + sGv.y), s1 = cell_sum(s1v.x + s1v.y);
   if (a.boost) {
     const float g2 = gam * gam;
     sI *= g2 * g2;
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     }
     __syncthreads();
     const int64_t cl = tile * CPB + lane;
-    if (warp == cell_warp<T>(tile, a.n_cells) && cl < a.n_cells) {
+    if (warp == cell_warp(tile, a.n_cells) && cl < a.n_cells) {
       float2 r = bcast(0.0f);
       if (a.kind[cl] == RT_CELL_INTERIOR) {
         float ql = 0.0f;
@@ -591,10 +591,10 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
     float *out = a.I_out + (size_t)c * RS;
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
-      const float4 xy = load_again(qd.xy + sub + T * i), zw = load_again(qd.zw + sub + T * i);
+      const float4 xy = load_again(qd.xy + sub + KT * i), zw = load_again(qd.zw + sub + KT * i);
       float2 na, nb;
       if (bnd) {
-        const float4 t = reinterpret_cast<const float4 *>(I0)[sub + T * i];
+        const float4 t = reinterpret_cast<const float4 *>(I0)[sub + KT * i];
         na = pfma(mf, psub(IA[i], make_float2(t.x, t.y)), IA[i]);
         nb = pfma(mf, psub(IB[i], make_float2(t.z, t.w)), IB[i]);
       } else {
@@ -607,11 +607,11 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
         nb = pmul(pfma(IB[i], GB3, QQ), prcpf(pmul(GB3, pfma(XS, GB, one))));
       }
       if (live)
-        reinterpret_cast<float4 *>(out)[sub + T * i] = make_float4(na.x, na.y, nb.x, nb.y);
+        reinterpret_cast<float4 *>(out)[sub + KT * i] = make_float4(na.x, na.y, nb.x, nb.y);
       float2 wa = bcast(a.w_uni), wb = wa;
       if (!uw) {
         wa = make_float2(zw.z, zw.w);
-        wb = __ldg(qd.wb + sub + T * i);
+        wb = __ldg(qd.wb + sub + KT * i);
       }
       const float2 da = pmul(wa, psub(IA[i], na)), db = pmul(wb, psub(IB[i], nb));
       dea = (dea + da.x) + da.y;
@@ -625,14 +625,14 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
       const float4 n = load_again(tdir);
       float2 nt;
       if (bnd) {
-        nt = pfma(mf, psub(IT, reinterpret_cast<const float2 *>(I0)[2 * T * NQ + sub]), IT);
+        nt = pfma(mf, psub(IT, reinterpret_cast<const float2 *>(I0)[2 * KT * NQ + sub]), IT);
       } else {
         const float bn = fmaf(vx, n.x, fmaf(vy, n.y, vz * n.z));
         const float2 G = make_float2(1.0f - bn, 1.0f + bn);
         const float2 G3 = pmul(pmul(G, G), G);
         nt = pmul(pfma(IT, G3, QQ), prcpf(pmul(G3, pfma(XS, G, one))));
       }
-      if (live) reinterpret_cast<float2 *>(out)[2 * T * NQ + sub] = nt;
+      if (live) reinterpret_cast<float2 *>(out)[2 * KT * NQ + sub] = nt;
       const float2 w = uw ? bcast(a.w_uni) : __ldg(W2);
       const float2 d = pmul(w, psub(IT, nt));
       dea += d.x;
@@ -646,14 +646,14 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   if (SMALL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   {
     const float v[4] = {dea + deb, dfx, dfy, dfz};
-    team_store4<T>(v, sub, lc, sh.sum);
+    cell_store4(v, sub, lc, sh.sum);
     if (sub == 0) sh.bad[lc] = bad;
   }
   __syncthreads();
 
   // ---------------- phase D: gas exchange, one lane per cell
   const int64_t cl = tile * CPB + lane;
-  if (warp == cell_warp<T>(tile, a.n_cells) && cl < a.n_cells) {
+  if (warp == cell_warp(tile, a.n_cells) && cl < a.n_cells) {
     unsigned b = sh.bad[lane];
     if (!isfinite(sh.sum[0][lane])) b |= ST_NONFINITE;
     gas_exchange<float, MOVING>(a, cl, stage.gas->gs[lane], stage.gas->gd[lane], sh.sum[0][lane],
@@ -661,28 +661,28 @@ __global__ void __launch_bounds__(CPB * T, quad_blocks<NQ, TAIL, T, SMALL>())
   }
 }
 
-template <int NQ, bool TAIL, int T, bool MOVING, bool SMALL>
+template <int NQ, bool TAIL, bool MOVING, bool SMALL>
 cudaError_t launch_quad_as(rt_state *s, const StepArgs<float> &a, unsigned blocks) {
   const int cap = stage_cap(s->max_block_slots);
   const float4 *xy = reinterpret_cast<const float4 *>(s->d_qdir);
   const int Q = s->n_angles / 4;
   const QuadDir qd{xy, xy + Q, reinterpret_cast<const float2 *>(xy + 2 * Q)};
-  auto *k = a.float_quartic ? quad_step_kernel<NQ, TAIL, T, MOVING, false, SMALL>
-                            : quad_step_kernel<NQ, TAIL, T, MOVING, true, SMALL>;
+  auto *k = a.float_quartic ? quad_step_kernel<NQ, TAIL, MOVING, false, SMALL>
+                            : quad_step_kernel<NQ, TAIL, MOVING, true, SMALL>;
   const cudaError_t e =
-      launch_carved(k, blocks, CPB * T, stage_bytes(cap, MOVING), quad_blocks<NQ, TAIL, T, SMALL>(),
+      launch_carved(k, blocks, NT, stage_bytes(cap, MOVING), quad_blocks<NQ, TAIL, SMALL>(),
                     sizeof(QuadShared), SMALL, s->stream, a, qd, cap);
   if (e != cudaSuccess) return e;
   s->launches++;
   return cudaGetLastError();
 }
 
-template <int NQ, bool TAIL, int T, bool MOVING>
+template <int NQ, bool TAIL, bool MOVING>
 cudaError_t launch_quad(rt_state *s, double dt, const StepIO &io) {
   const StepArgs<float> a = step_args<float>(s, dt, io);
   const unsigned blocks = (unsigned)((s->n_cells + CPB - 1) / CPB);
-  return blocks <= 2 * 152 ? launch_quad_as<NQ, TAIL, T, MOVING, true>(s, a, blocks)
-                           : launch_quad_as<NQ, TAIL, T, MOVING, false>(s, a, blocks);
+  return blocks <= 2 * 152 ? launch_quad_as<NQ, TAIL, MOVING, true>(s, a, blocks)
+                           : launch_quad_as<NQ, TAIL, MOVING, false>(s, a, blocks);
 }
 
 template <typename M, bool MOVING>
@@ -714,13 +714,13 @@ cudaError_t dispatch_pairs(rt_state *s, double dt, const StepIO &io) {
 // tail pair when m is odd.
 template <bool MOVING> cudaError_t dispatch_quads(rt_state *s, double dt, const StepIO &io) {
   switch (s->n_angles / 16) {
-    case 2: return launch_quad<1, false, 8, MOVING>(s, dt, io);
-    case 3: return launch_quad<1, true, 8, MOVING>(s, dt, io);
-    case 4: return launch_quad<2, false, 8, MOVING>(s, dt, io);
-    case 5: return launch_quad<2, true, 8, MOVING>(s, dt, io);
-    case 6: return launch_quad<3, false, 8, MOVING>(s, dt, io);
-    case 7: return launch_quad<3, true, 8, MOVING>(s, dt, io);
-    case 8: return launch_quad<4, false, 8, MOVING>(s, dt, io);
+    case 2: return launch_quad<1, false, MOVING>(s, dt, io);
+    case 3: return launch_quad<1, true, MOVING>(s, dt, io);
+    case 4: return launch_quad<2, false, MOVING>(s, dt, io);
+    case 5: return launch_quad<2, true, MOVING>(s, dt, io);
+    case 6: return launch_quad<3, false, MOVING>(s, dt, io);
+    case 7: return launch_quad<3, true, MOVING>(s, dt, io);
+    case 8: return launch_quad<4, false, MOVING>(s, dt, io);
     default: return cudaErrorInvalidValue;
   }
 }

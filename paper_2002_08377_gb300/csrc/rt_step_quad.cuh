@@ -1,5 +1,5 @@
-// The float step over quad rows: T threads per cell, thread `sub` owning the
-// quads sub + T i (i < NQ) of a row, each as two packed FP32 units: (p, p+1) and
+// The float step over quad rows: KT threads per cell, thread `sub` owning the
+// quads sub + KT i (i < NQ) of a row, each as two packed FP32 units: (p, p+1) and
 // their antipodes.
 #pragma once
 
@@ -17,20 +17,10 @@ template <int NQ, bool TAIL, bool MOVING> constexpr int quad_unroll() {
   return NQ == 1 ? 3 : (TAIL && NQ == 2) || (MOVING && NQ > 2) ? 1 : 2;
 }
 __device__ __forceinline__ float2 bcast(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 pmin0(float2 v) {
-  return make_float2(fminf(v.x, 0.0f), fminf(v.y, 0.0f));
-}
 __device__ __forceinline__ float2 pmax0(float2 v) {
   return make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f));
 }
 __device__ __forceinline__ float2 prcpf(float2 v) { return make_float2(rcp(v.x), rcp(v.y)); }
-
-// Sum over a cell's T threads, in every one of them.
-template <int T> __device__ __forceinline__ float team_sum(float v) {
-#pragma unroll
-  for (int o = T / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // The direction table of the quads, each array contiguous over them:
 // (nx0, nx1, ny0, ny1), (nz0, nz1, wa0, wa1), (wb0, wb1).
@@ -63,7 +53,7 @@ template <int NQ> struct QuadSums {
 // CHUNK > 0 (meshes that leave the SMs mostly idle): the rows of CHUNK faces are
 // loaded before the first one's arithmetic, the last chunk filled up with its
 // last face's loads.
-template <int NQ, bool TAIL, int T, bool MOVING, int CHUNK>
+template <int NQ, bool TAIL, bool MOVING, int CHUNK>
 __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr, int k0, int k1,
                                            const float *I_in, int RS, int sub,
                                            const float2 (&NX)[NQ], const float2 (&NY)[NQ],
@@ -84,8 +74,8 @@ __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr
     const float *row = I_in + (size_t)nb * RS;
     const float4 *q = reinterpret_cast<const float4 *>(row) + sub;
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) f.v[i] = q[T * i];
-    f.vt = TAIL ? reinterpret_cast<const float2 *>(row)[2 * T * NQ + sub] : bcast(0.0f);
+    for (int i = 0; i < NQ; ++i) f.v[i] = q[KT * i];
+    f.vt = TAIL ? reinterpret_cast<const float2 *>(row)[2 * KT * NQ + sub] : bcast(0.0f);
   };
   auto add = [&](const Face &f) {
     const float4 s = f.s;
@@ -131,31 +121,19 @@ __device__ __forceinline__ void quad_faces(const SlotF *slot, const int32_t *nbr
   }
 }
 
-// The sums of v[0..3] over a cell's T threads, written to out[k][lc] (the
-// halving exchange of cell_reduce4; each value in a fixed order).
-template <int T>
-__device__ __forceinline__ void team_store4(const float (&v)[4], int sub, int lc,
+// The sums of v[0..3] over a cell's 8 threads, written to out[k][lc] (a halving
+// exchange; each value in a fixed order).
+__device__ __forceinline__ void cell_store4(const float (&v)[4], int sub, int lc,
                                             float (*out)[CPB]) {
-  if constexpr (T == 1) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) out[k][lc] = v[k];
-  } else {
-    constexpr int h = T / 2;
-    const bool hi = sub & h;
-    float a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
-    a += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], h);
-    b += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], h);
-    if constexpr (T == 2) {
-      out[hi ? 2 : 0][lc] = a;
-      out[hi ? 3 : 1][lc] = b;
-    } else {
-      const bool odd = sub & (h / 2);
-      float c = odd ? b : a;
-      c += __shfl_xor_sync(0xffffffffu, odd ? a : b, h / 2);
-      if constexpr (T == 8) c += __shfl_xor_sync(0xffffffffu, c, 1);
-      if (T == 4 || !(sub & 1)) out[(hi ? 2 : 0) + (odd ? 1 : 0)][lc] = c;
-    }
-  }
+  static_assert(KT == 8, "three exchanges");
+  const bool hi = sub & 4, odd = sub & 2;
+  float a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
+  a += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 4);
+  b += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 4);
+  float c = odd ? b : a;
+  c += __shfl_xor_sync(0xffffffffu, odd ? a : b, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  if (!(sub & 1)) out[(hi ? 2 : 0) + (odd ? 1 : 0)][lc] = c;
 }
 
 }  // namespace step
