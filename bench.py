@@ -40,13 +40,13 @@ UNIT = "cell-angle updates/s"
 # capture (dram__bytes_read.sum + dram__bytes_write.sum, one launch, one
 # pass); valid while the step kernel's device source has the recorded hash
 # (else reported as null).  FP32: the 256^3 linear-wave launch itself
-# (12.42 GB read + 6.15 GB written).  FP64: the 128^3 linear-wave launch
-# (12.52 + 1.49 GB, mostly the flux-coefficient table) scaled by the cell
-# count to 256^3 (the table, the rows and the gas all grow with the cells),
-# taken when only the float instantiations' code differed from today's.
-NCU_TRAFFIC = {("waves", 16777216, "fp32"): 18.57e9,
-               ("waves", 16777216, "fp64"): 14.01e9 * 8}
-NCU_SOURCE_SHA = "3210b6995f7435eb"
+# (12.44 GB read + 6.19 GB written).  FP64: the 128^3 linear-wave launch
+# (13.87 + 1.47 GB, mostly the flux-coefficient table) scaled by the cell
+# count to 256^3 (the tables, the rows and the gas all grow with the cells).
+# Taken at source d660daf06b0fd4f3, from which only comments differ.
+NCU_TRAFFIC = {("waves", 16777216, "fp32"): 18.63e9,
+               ("waves", 16777216, "fp64"): 15.34e9 * 8}
+NCU_SOURCE_SHA = "5eef700e7cec9c18"
 # FP64 arithmetic peak when the DGEMM probe cannot run: the nominal dense
 # FP64 FMA rate of the GPU.
 FP64_NOMINAL_GFLOPS = 1250.0
@@ -811,7 +811,7 @@ def main():
                 "ms_per_step": head["fp32_float_quartic"]["ms_per_step"],
                 "frac": head["fp32_float_quartic"]["roofline"]["frac"],
                 "note": "the FP32 state with float_quartic = 1 (temperature solved in float in "
-                        "every lane); the headline solves it in double"},
+                        "every lane); the headline refines that root"},
             "fp64": {"value": r64["value"], "ms_per_step": r64["ms_per_step"],
                      "steps": r64["steps"], "dtype": "f64", "launches": r64["launches"],
                      "device_bytes": r64["device_bytes"], "roofline": r64["roofline"],

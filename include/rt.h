@@ -62,9 +62,10 @@ typedef enum {
 
 typedef enum {
   RT_FP64 = 0, /* every quantity in double precision                          */
-  RT_FP32 = 1  /* intensities, face geometry and the transport sweep in float;
-                  the temperature quartic, the gas energy/momentum exchange
-                  and the conservation sums in double                         */
+  RT_FP32 = 1  /* intensities, face geometry, the transport sweep and the
+                  coefficients of the temperature equation in float; the gas
+                  energy/momentum exchange and the conservation sums in double;
+                  the root of the temperature equation: rt_params.float_quartic */
 } rt_precision;
 
 typedef enum {
@@ -138,7 +139,10 @@ typedef enum { RT_FIRST_ORDER = 0, RT_VAN_LEER = 1 } rt_integrator;
  * speed of light of the transport, c the true one (enters the gas coupling
  * and the moments).  r_gas = k_B / (mu m_p); c_v = r_gas / (gamma_gas - 1).
  * cfl scales the Courant step dt = cfl * min V^(1/3) / (cbar + |w|).
- * newton_max_iter <= 0 selects 64.  boost selects the frequency ratio of the
+ * newton_max_iter <= 0 selects 64; a step in which a cell's Newton iteration has not
+ * converged within it returns RT_ERR_NONCONV (FP32 states: a cell whose float
+ * iteration has not is solved again in double with the same limit first, unless
+ * float_quartic = 1).  boost selects the frequency ratio of the
  * comoving transformation (Sec. 2.3), Gamma_a = gamma (1 - v . n_a / c):
  * 0 takes gamma = 1 (first order in v/c), 1 the Lorentz factor
  * gamma = (1 - v^2 / c^2)^(-1/2) of the cell's frame velocity (all orders;
@@ -165,14 +169,14 @@ typedef enum { RT_FIRST_ORDER = 0, RT_VAN_LEER = 1 } rt_integrator;
  * plain_launches = 0 (the default) lets rt_run / rt_launch replay a CUDA
  * graph of RT_GRAPH_STEPS steps captured on the state's stream (see rt_run);
  * 1 launches every kernel from the host.  Both give identical results.
- * float_quartic (RT_FP32 states only, ignored for RT_FP64): 0, the default,
- * solves the gas temperature equation of Eq. (com rad thermal disc) to
- * double accuracy, as the precision split of RT_FP32 states says: the emission
- * it gives is the one that coefficients formed in double from the float angular
- * sums and Newton in double give, rounded to float (found in float and refined
- * by pairs of floats; where that is not certain, by the double Newton itself);
- * 1 solves it in float alone (faster; coefficients outside float range still
- * take the double solve), so the temperature carries float rounding.
+ * float_quartic (RT_FP32 states only, ignored for RT_FP64): in both
+ * settings the coefficients of the gas temperature equation of Eq. (com rad
+ * thermal disc) are formed in float, from the float angular sums and opacities,
+ * and the emission is evaluated in float from a float temperature.  0, the
+ * default, takes the float nearest to the root of that equation (the float root
+ * refined by one Newton step with its residual to double accuracy); 1 takes the
+ * float Newton's root as it is, a few float roundings away (faster).
+ * Coefficients or emissions outside float range take the double solve in both.
  * hydro = 1 lets the state evolve the gas by the Euler equations as well
  * (rt_hydro_step, rt_radhydro_step: Sec. 2, radiation subcycled under a
  * hydro step); it needs face_offset, a static mesh (face_w NULL or zero),
@@ -187,7 +191,7 @@ typedef struct {
   int32_t gcl;             /* 0 or 1, see above */
   int32_t plain_launches;  /* 0: multi-step calls replay captured graphs; 1: plain launches */
   double beta_P, beta_J, T_ref; /* see above */
-  int32_t float_quartic;   /* RT_FP32 only: 0 temperature solve in double, 1 in float */
+  int32_t float_quartic;   /* RT_FP32 only: 0 temperature root refined, 1 float root as it is */
   int32_t hydro;           /* 1: the state also evolves the gas dynamics (rt_hydro_step) */
 } rt_params;
 

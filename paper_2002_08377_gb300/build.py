@@ -14,9 +14,10 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librt_gb300.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["rt_api.cu", "rt_step.cu", "rt_step64.cu", "rt_step_cell.cu", "rt_transport.cu", "rt_aux.cu", "rt_adjoint.cu", "rt_noalloc.cu",
-           "rt_recon.cu", "rt_groups.cu", "rt_hydro.cu"]
-# per-file flags: the gas dynamics round as their plain formulas (no FMA contraction)
+SOURCES = ["rt_api.cu", "rt_step.cu", "rt_step64.cu", "rt_step_cell.cu", "rt_transport.cu",
+           "rt_aux.cu", "rt_adjoint.cu", "rt_noalloc.cu", "rt_recon.cu", "rt_groups.cu",
+           "rt_hydro.cu"]
+# per-file flags: the gas dynamics contract no further FMAs than the ones they write out
 FILE_FLAGS = {"rt_hydro.cu": ["--fmad=false"]}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code is compiled without FMA contraction so that x86 and Arm hosts

@@ -423,12 +423,12 @@ __global__ void __launch_bounds__(kThreads) group_source_kernel(const GroupArgs<
 // pair / quad map).  The group of pair p is p / Hb, and every sum is kept
 // per group (unused groups stay zero).  Float states find the root of the
 // temperature equation in float in all 8 lanes of a cell, from float copies
-// of the group opacities; by default one lane per cell then refines it by a
-// Newton step in double between two block barriers and forms the groups' q_j
-// (float_quartic = 1 keeps the float root, with no barrier); where a float
-// result is not finite the double chain runs instead.  Double states solve
-// it one lane per cell in double between two barriers.  The gas exchange is
-// one lane per cell in double after a barrier, as in the grey step.
+// of the group opacities, and by default refine it there in float pairs
+// (step::refine_quartic; float_quartic = 1 keeps the float root).  Where a cell of the
+// block needs more (found by a block vote), one lane per cell takes the Newton step in
+// double, or the double chain where a float result is not finite, between two barriers.
+// Double states solve it one lane per cell in double between two barriers.  The gas
+// exchange is one lane per cell in double after a barrier, as in the grey step.
 template <typename R> struct TileShared {
   double s[CPB][kTileGroups][3];  // S_I, S_G, S_1 per group
   R q[CPB][kTileGroups];

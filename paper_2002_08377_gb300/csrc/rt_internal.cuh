@@ -47,8 +47,8 @@ constexpr int kMomTab = 12;
 
 // The step kernel works on blocks of CPB consecutive (internal) cells.
 constexpr int CPB = 32;
-// Face slots of one block of CPB cells that the float QuadMap kernel stages
-// in shared memory at most; meshes with more take the PairMap kernel.
+// Face slots of one block of CPB cells that the float kernels of quad rows and of at
+// most 8 angles stage in shared memory at most; meshes with more take the tile kernel.
 constexpr int STAGE_SLOTS = 1024;
 
 // Per-cell constant gas data: rho, the absorption / scattering coefficients

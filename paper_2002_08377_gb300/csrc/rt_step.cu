@@ -22,10 +22,11 @@
 // What bounds it: latency.  A block's time is the sum of its phases' waits (its
 // stage, the gathers of the neighbour rows from L1 / L2, the double gas update),
 // which four resident blocks overlap only in part: no unit is saturated (96^3 x
-// 64: issue 52 %, L1 data pipe 60 %, DRAM 26 %).  Hence the L2 prefetch one wave
-// ahead (11 %), one block barrier only, packed FP32 on (p, p+1) throughout,
-// registers capped at 64 so that four blocks fit, and L1 given what shared memory
-// leaves.  Per step, before (double refinement between two barriers, no
+// 80: issue 59 %, L1 data pipe 62 %, DRAM 24 %, FP64 10 %; of the 12 cycles between a
+// warp's instructions 4.5 wait for loads, 1.9 for results, 1.5 at the barrier).  Hence
+// the L2 prefetch one wave ahead (11 %), one block barrier only, packed FP32 on (p, p+1)
+// throughout, registers capped at 64 so that four blocks fit, and L1 given what shared
+// memory leaves.  Per step, before (double refinement between two barriers, no
 // prefetch) and now, rows bit for bit the same: 96^3 x 80 static 558 -> 493 us,
 // 128^3 x 80 1290 -> 1131, 64^3 x 96 211 -> 168, 100^3 x 48 moving 511 -> 484.
 // Staging every row a tile reads in shared memory by bulk copies (128^3 x 64:
@@ -50,8 +51,9 @@ struct Shared {
 };
 
 // One block of CPB cells of a state whose rows are in the pair layout: the
-// phases of the quad kernel, slots read from global memory, the temperature
-// refined in double by one lane per cell between two block barriers.
+// phases of the quad kernel, slots read from global memory, the temperature refined by
+// one lane per cell between two block barriers (source_q_refined; float_quartic = 1: the
+// float root in every lane, no barrier).
 template <typename M, bool MOVING>
 __global__ void __launch_bounds__(NT, min_blocks<M::PPT>()) step_kernel(const StepArgs<float> a) {
   __shared__ Shared sh;

@@ -45,9 +45,9 @@ struct SharedGas {
   GasDyn gd[CPB];
 };
 
-// One tile's inputs staged in shared memory by the float QuadMap kernel:
-// the tile's face slots (static meshes: with the neighbour index in w), the
-// neighbour indices (moving meshes) and the gas records.
+// One tile's inputs staged in shared memory by the float kernels of quad rows: the
+// tile's face slots (static meshes: with the neighbour index in w), the neighbour
+// indices (moving meshes) and, for quad_step_kernel, the gas records.
 struct StageView {
   SlotF *slot;
   int32_t *nbr;
