@@ -91,6 +91,24 @@ def test_roots_near_a_midpoint(probe, off):
         assert took.mean() > 0.99
 
 
+@pytest.mark.parametrize("shift", [0, 40, 55, 65, 80])
+def test_small_energy_densities(probe, shift):
+    """The same equations in units of energy density 2^shift times larger: accepted down
+    to g = 2^-98 and beta = 2^-100, with the same floats as the double step."""
+    rng = np.random.default_rng(3)
+    n = 1 << 21
+    T = np.exp2(rng.uniform(0, 12, n))
+    beta = np.exp2(rng.uniform(-17.9, 0, n)) * (1 + rng.uniform(-1, 1, n) * 2.0 ** -24)
+    alpha = (beta / T ** 3 * np.exp2(rng.uniform(-10, 10, n))).astype(np.float32)
+    beta = beta * 2.0 ** -shift
+    alpha = (alpha * np.float32(2.0 ** -(shift // 2))) * np.float32(2.0 ** -(shift - shift // 2))
+    g = (alpha.astype(np.float64) * T ** 4 + beta * T).astype(np.float32)
+    T0 = T * (1 + 0.1 * rng.uniform(-1, 1, n))
+    quick, took, full = probe(alpha, beta, g, T0, 1e-4)
+    assert np.array_equal(quick[took].view(np.uint32), full[took].view(np.uint32))
+    assert (~took).mean() < 1e-4
+
+
 def test_guard_limits(probe):
     """Powers of two as roots, and scales at and past the guards' limits."""
     rng = np.random.default_rng(9)
