@@ -57,9 +57,11 @@ __device__ __forceinline__ bool refine_quartic(float alpha, double beta, float b
   *T = Tr;
   const float e = (T0 - Tr) - d;  // the unrounded result minus Tr
   const unsigned b = __float_as_uint(Tr);
-  const float half = __uint_as_float((b & 0x7f800000u) - (24u << 23));  // half an ulp of Tr
-  return ok && fabsf(fabsf(e) - half) > Tr * 0x1p-40f && (b & 0x007fffffu) != 0 &&
-         fabsf(d) <= 3e-7f * Tr;
+  // half the distance to the next float on e's side (below a power of two half of that
+  // above it)
+  const unsigned lower = (b & 0x007fffffu) == 0 && e < 0.0f ? 25u : 24u;
+  const float half = __uint_as_float((b & 0x7f800000u) - (lower << 23));
+  return ok && fabsf(fabsf(e) - half) > Tr * 0x1p-40f && fabsf(d) <= 3e-7f * Tr;
 }
 
 // The temperature equation of a float state's cell in float: the

@@ -5,8 +5,8 @@ says it does.  The probe is compiled from the kernels' own header.
 
 Equations over the whole range of the guards, beta rounding up and down to float,
 one of the two terms dominant or both alike, temperatures near and far from the
-root, and roots laid next to the midpoint of two floats and onto powers of two,
-where it must decline."""
+root, roots laid next to the midpoint of two floats, where it must decline, and onto
+powers of two, whose neighbour below is half as far as the one above."""
 import ctypes
 import os
 import subprocess
@@ -69,6 +69,30 @@ def test_accepted_roots_equal_the_double_step(probe, spread, tol):
     assert (~took).mean() < 1e-4
 
 
+@pytest.mark.parametrize("off", [0.0, 2.0 ** -30, -2.0 ** -30, 2.0 ** -25, -2.0 ** -25,
+                                 -2.0 ** -25 * (1 - 2.0 ** -13), -2.0 ** -25 * (1 + 2.0 ** -13),
+                                 2.0 ** -24 * (1 - 2.0 ** -13), 2.0 ** -24 * (1 + 2.0 ** -13),
+                                 -2.0 ** -24])
+def test_roots_at_powers_of_two(probe, off):
+    """The root a power of two (uniform gas at T = 1) times (1 + off): accepted unless it
+    lies next to a midpoint, 2^-24 above and 2^-25 below."""
+    rng = np.random.default_rng(11)
+    n = 1 << 18
+    two = np.exp2(rng.integers(-8, 9, n).astype(np.float64))
+    T = two * (1 + off)
+    alpha = (np.exp2(rng.uniform(-4, 4, n)) / T ** 3).astype(np.float32)
+    g = (alpha.astype(np.float64) * T ** 4 * rng.uniform(1.5, 8.0, n)).astype(np.float32)
+    beta = (g - alpha.astype(np.float64) * T ** 4) / T
+    T0 = two.astype(np.float32)
+    T0 = np.where(rng.uniform(size=n) < 0.3, np.nextafter(T0, np.float32(0)), T0)
+    quick, took, full = probe(alpha, beta, g, T0, 0.0)
+    assert np.array_equal(quick[took].view(np.uint32), full[took].view(np.uint32))
+    if off == -2.0 ** -25:
+        assert not took.any()
+    else:
+        assert took.all()
+
+
 @pytest.mark.parametrize("off", [0.0, 2.0 ** -44, -2.0 ** -44, 2.0 ** -41, -2.0 ** -41,
                                  2.0 ** -39, -2.0 ** -39, 2.0 ** -30])
 def test_roots_near_a_midpoint(probe, off):
@@ -124,5 +148,3 @@ def test_guard_limits(probe):
     quick, took, full = probe(alpha[ok], beta[ok], g[ok], T[ok].astype(np.float32), 0.0)
     assert took.any() and not took.all()
     assert np.array_equal(quick[took].view(np.uint32), full[took].view(np.uint32))
-    two = (quick[took].view(np.uint32) & 0x007fffff) == 0
-    assert not two.any()
