@@ -43,10 +43,11 @@ UNIT = "cell-angle updates/s"
 # (12.44 GB read + 6.19 GB written).  FP64: the 128^3 linear-wave launch
 # (13.87 + 1.47 GB, mostly the flux-coefficient table) scaled by the cell
 # count to 256^3 (the tables, the rows and the gas all grow with the cells).
-# Taken at source d660daf06b0fd4f3, from which only comments differ.
+# Taken at source d660daf06b0fd4f3, from which comments and the ranges of the
+# in-lane temperature refinement differ (no memory traffic).
 NCU_TRAFFIC = {("waves", 16777216, "fp32"): 18.63e9,
                ("waves", 16777216, "fp64"): 15.34e9 * 8}
-NCU_SOURCE_SHA = "5eef700e7cec9c18"
+NCU_SOURCE_SHA = "93bc2d2390ba47a3"
 # FP64 arithmetic peak when the DGEMM probe cannot run: the nominal dense
 # FP64 FMA rate of the GPU.
 FP64_NOMINAL_GFLOPS = 1250.0

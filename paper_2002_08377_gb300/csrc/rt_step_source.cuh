@@ -61,7 +61,8 @@ __device__ __forceinline__ bool refine_quartic(float alpha, double beta, float b
   // above it)
   const unsigned lower = (b & 0x007fffffu) == 0 && e < 0.0f ? 25u : 24u;
   const float half = __uint_as_float((b & 0x7f800000u) - (lower << 23));
-  return ok && fabsf(fabsf(e) - half) > Tr * 0x1p-40f && fabsf(d) <= 3e-7f * Tr;
+  return (ok && fabsf(fabsf(e) - half) > Tr * 0x1p-40f && fabsf(d) <= 3e-7f * Tr) ||
+         (g == 0.0f && T0 == 0.0f);  // a dark vacuum: T = 0 exactly
 }
 
 // The temperature equation of a float state's cell in float: the

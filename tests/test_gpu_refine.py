@@ -133,6 +133,17 @@ def test_small_energy_densities(probe, shift):
     assert (~took).mean() < 1e-4
 
 
+def test_vacuum(probe):
+    """The root 0 of a dark cell without energy, opaque or not."""
+    rng = np.random.default_rng(13)
+    n = 1 << 12
+    alpha, beta = np.exp2(rng.uniform(-20, 20, n)), np.exp2(rng.uniform(-90, 20, n))
+    alpha[::2] = 0.0
+    zero = np.zeros(n)
+    quick, took, full = probe(alpha, beta, zero, zero, 0.0)
+    assert took.all() and not quick.any() and not full.any()
+
+
 def test_guard_limits(probe):
     """Powers of two as roots, and scales at and past the guards' limits."""
     rng = np.random.default_rng(9)
