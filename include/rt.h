@@ -180,8 +180,8 @@ typedef enum { RT_FIRST_ORDER = 0, RT_VAN_LEER = 1 } rt_integrator;
  * hydro = 1 lets the state evolve the gas by the Euler equations as well
  * (rt_hydro_step, rt_radhydro_step: Sec. 2, radiation subcycled under a
  * hydro step); it needs face_offset, a static mesh (face_w NULL or zero),
- * n_groups 1, gcl 0 and constant opacities, and adds about 150 bytes per
- * face and 230 per cell of device memory. */
+ * n_groups 1, gcl 0 and constant opacities, and adds about 300 bytes per
+ * face and 310 per cell of device memory. */
 typedef struct {
   double cbar, c, a_rad, gamma_gas, r_gas, cfl;
   int32_t precision;       /* rt_precision */
